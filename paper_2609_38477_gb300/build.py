@@ -11,7 +11,7 @@ ROOT = os.path.dirname(PKG)
 CSRC = os.path.join(PKG, "csrc")
 BUILD = os.path.join(ROOT, "_build")
 LIB = os.path.join(PKG, "libseedq.so")
-SOURCES = ["plan.cu", "decode.cu", "gemv.cu", "encode.cu", "importance.cu", "container.cpp"]
+SOURCES = ["plan.cu", "decode.cu", "gemv.cu", "encode.cu", "encode_screen.cu", "importance.cu", "container.cpp"]
 # Every header a translation unit may include: an edit to any of them rebuilds all objects.
 HEADERS = sorted(glob.glob(os.path.join(CSRC, "*.cuh")) + glob.glob(os.path.join(CSRC, "*.h")) +
                  glob.glob(os.path.join(ROOT, "include", "*.h")))

@@ -20,8 +20,11 @@
 // (2^{1-S}) are restored exactly in the exponent arithmetic; Gaussian
 // elimination commutes with scaling by powers of two.
 //
-// Work split: one warp per block, lanes striding over the seeds, then a warp
-// reduction on (error, seed).
+// Two routes give the same bits.  The screened search (encode_screen.cu)
+// evaluates only the seeds that can still win and is taken by all but the
+// smallest calls.  The exhaustive kernels here evaluate every seed: one warp
+// per block, lanes striding over the seeds, then a warp reduction on (error,
+// seed); they also serve calls for which no scratch memory is left.
 //
 // The fp64 pipe is the bottleneck (a small fraction of the integer pipes'
 // rate), so every step whose result is exact is done with integer
@@ -31,217 +34,46 @@
 // patterns; the quotients of the solve are exact IEEE divisions done with
 // 64-bit integer arithmetic (div_rn).  Only the rounded sums and products of
 // the solve and the error run on the fp64 pipe.
-#include "seedq_internal.cuh"
+#include "encode_core.cuh"
 
 namespace seedq {
 
 constexpr int kEncWarps = 8;
 
-// Power of two 2^e as a double (|e| well inside the normal range).
-__device__ __forceinline__ double pow2d(int e) { return __longlong_as_double((long long)(1023 + e) << 52); }
-
-// The double equal to the integer +-mag * 2^e (mag < 2^63), built from bits.
-__device__ __forceinline__ double exact_d(bool neg, unsigned long long mag, int e) {
-  if (mag == 0) return 0.0;
-  const int msb = 63 - __clzll((long long)mag);
-  const unsigned long long mant = (msb <= 52 ? (mag << (52 - msb)) : (mag >> (msb - 52))) & ((1ull << 52) - 1);
-  return __longlong_as_double((long long)(((unsigned long long)neg << 63) |
-                                          ((unsigned long long)(1023 + msb + e) << 52) | mant));
-}
-__device__ __forceinline__ double i2d(long long v) {
-  return exact_d(v < 0, (unsigned long long)(v < 0 ? -v : v), 0);
-}
-// |bits| of a double, as an integer whose order is the order of magnitudes.
-__device__ __forceinline__ unsigned long long mag_bits(double d) {
-  return (unsigned long long)__double_as_longlong(d) & 0x7fffffffffffffffull;
-}
-// d * 2^e for d normal or zero (exponent field shift).
-__device__ __forceinline__ double scale2(double d, int e) {
-  const long long b = __double_as_longlong(d);
-  return (b & 0x7fffffffffffffffll) == 0 ? d : __longlong_as_double(b + ((long long)e << 52));
-}
-
-// All k round-half-even values of x_j * 2^e lie in [-8, 7], i.e. every
-// x_j * 2^e lies in [-8.5, 7.5) (compared as bit patterns: exact).
-template <int K>
-__device__ __forceinline__ bool fits(const double (&x)[K], int e) {
-  const unsigned long long lim_neg = (unsigned long long)__double_as_longlong(8.5);
-  const unsigned long long lim_pos = (unsigned long long)__double_as_longlong(7.5);
-  bool ok = true;
-#pragma unroll
-  for (int j = 0; j < K; ++j) {
-    const double v = scale2(x[j], e);
-    const unsigned long long b = (unsigned long long)__double_as_longlong(v);
-    ok = ok && ((b >> 63) ? ((b & 0x7fffffffffffffffull) <= lim_neg) : (b < lim_pos));
-  }
-  return ok;
-}
+// Whether a call takes the screened search (encode_screen.cu).  Its tables and
+// thresholds are a fixed cost (about 150 us), which 255 seeds of few
+// coefficients do not repay on small calls; measured at (8, 3), exhaustive
+// against screened: 84 / 163 us at 100 blocks, 162 / 182 at 2000, 1214 / 194
+// at 20000; at (8, 6) 340 / 322 at 100; at (10, 2) 176 / 164 at 100.
+static bool screened(int S, int K, int64_t nblocks) { return S > 8 || K > 3 || nblocks > 2048; }
 
 // Search all seeds of one block (w: 8 weights) for the lane's share of seeds.
 // Returns the lane's best (error, seed, E, t) in the order of the scan.
-template <int K, bool kExactRhs>
+template <int K>
 __device__ __forceinline__ void search_block(int S, const uint64_t *tab, const float (&wf)[8], int lane,
                                              double &best, uint32_t &bseed, int &bE, int (&bt)[6]) {
-  // Each weight as +-mw * 2^ew with an integer mantissa (exact for floats).
-  double w[8];
-  bool wneg[8];
-  unsigned int wm[8];
-  int we[8];
-#pragma unroll
-  for (int i = 0; i < 8; ++i) {
-    w[i] = (double)wf[i];
-    const unsigned int fb = __float_as_uint(wf[i]);
-    const int ef = (int)((fb >> 23) & 255u);
-    wneg[i] = (fb >> 31) != 0;
-    wm[i] = (fb & 0x7fffffu) | (ef ? 0x800000u : 0u);
-    we[i] = (ef ? ef : 1) - 150;
-  }
-  // Right-hand side without rounding: when the weights' exponents lie within
-  // 11 of each other, every product |u| * mw (< 2^39) aligned to the smallest
-  // exponent stays below 2^50, so every partial sum of the eight is an integer
-  // below 2^53: each fp64 addition of the sequence is then exact, and the sum
-  // equals the integer sum (the caller picks this variant per block).
-  int emin = 1 << 20;
-#pragma unroll
-  for (int i = 0; i < 8; ++i)
-    if (wm[i]) emin = min(emin, we[i]);
-  if (emin == (1 << 20)) emin = 0;  // all weights zero
-  int wsh[8];
-#pragma unroll
-  for (int i = 0; i < 8; ++i) wsh[i] = wm[i] ? we[i] - emin : 0;
-  const uint32_t mask = (1u << S) - 1u;
-  const int h = 1 << (S - 1);
-  // Pivot threshold of the unscaled matrix: 1e-12 * 2^(2S-2), exact.
-  const unsigned long long thr = mag_bits(__dmul_rn(1e-12, pow2d(2 * S - 2)));
+  const BlockParts B(wf);
   best = __longlong_as_double(0x7ff0000000000000ll);  // +inf
   bseed = 0;
   bE = 0;
 #pragma unroll
   for (int j = 0; j < 6; ++j) bt[j] = 0;
-  const uint32_t nseeds = mask;  // seeds 1 .. 2^S - 1
+  const uint32_t nseeds = (1u << S) - 1u;  // seeds 1 .. 2^S - 1
   for (uint32_t s = 1 + lane; s <= nseeds; s += 32) {
     const uint64_t Q = tab[s & 255u] ^ tab[256 + ((s >> 8) & 255u)];
     int u[8][K];
-#pragma unroll
-    for (int i = 0; i < 8; ++i)
-#pragma unroll
-      for (int j = 0; j < K; ++j) u[i][j] = (int)((uint32_t)(Q >> (i * K + j)) & mask) - h;
-    // Normal equations (unscaled): A[p][q] exact integers, b[p] rounded in i order.
-    double A[K][K], b[K];
-#pragma unroll
-    for (int p = 0; p < K; ++p) {
-      if constexpr (kExactRhs) {
-        long long acc = 0;
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-          const long long pr = ((long long)u[i][p] * (long long)wm[i]) << wsh[i];
-          acc += wneg[i] ? -pr : pr;
-        }
-        b[p] = exact_d(acc < 0, (unsigned long long)(acc < 0 ? -acc : acc), emin);
-      } else {
-        double r = 0.0;
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-          // u * w is exact: built from the integer product of the mantissas.
-          const int ui = u[i][p];
-          const double prod = exact_d(wneg[i] != (ui < 0),
-                                      (unsigned long long)(ui < 0 ? -ui : ui) * wm[i], we[i]);
-          r = __dadd_rn(r, prod);
-        }
-        b[p] = r;
-      }
-#pragma unroll
-      for (int q = p; q < K; ++q) {
-        long long acc = 0;
-#pragma unroll
-        for (int i = 0; i < 8; ++i) acc += (long long)(u[i][p] * u[i][q]);
-        A[p][q] = i2d(acc);
-        A[q][p] = A[p][q];
-      }
-    }
-    // Gaussian elimination with partial pivoting (first row of largest |pivot|).
-    // Divisions are exact IEEE quotients on the integer pipes (div_rn), one
-    // reciprocal estimate per pivot, reused by the back substitution.
-    bool singular = false;
-    DivRecip Rp[K];
-#pragma unroll
-    for (int c = 0; c < K; ++c) {
-      int pr = c;
-      unsigned long long pv = mag_bits(A[c][c]);
-#pragma unroll
-      for (int r = c + 1; r < K; ++r) {
-        const unsigned long long v = mag_bits(A[r][c]);
-        if (v > pv) {
-          pv = v;
-          pr = r;
-        }
-      }
-      singular = singular || (pv < thr);
-#pragma unroll
-      for (int r = c + 1; r < K; ++r) {
-        if (pr == r) {
-#pragma unroll
-          for (int q = c; q < K; ++q) {
-            const double tmp = A[c][q];
-            A[c][q] = A[r][q];
-            A[r][q] = tmp;
-          }
-          const double tb = b[c];
-          b[c] = b[r];
-          b[r] = tb;
-        }
-      }
-      Rp[c] = div_recip(A[c][c]);
-#pragma unroll
-      for (int r = c + 1; r < K; ++r) {
-        const double f = div_rn(A[r][c], Rp[c]);
-#pragma unroll
-        for (int q = c + 1; q < K; ++q) A[r][q] = __dsub_rn(A[r][q], __dmul_rn(f, A[c][q]));
-        b[r] = __dsub_rn(b[r], __dmul_rn(f, b[c]));
-      }
-    }
-    if (singular) continue;
-    double x[K];
-#pragma unroll
-    for (int r = K - 1; r >= 0; --r) {
-      double sacc = b[r];
-#pragma unroll
-      for (int q = r + 1; q < K; ++q) sacc = __dsub_rn(sacc, __dmul_rn(A[r][q], x[q]));
-      x[r] = div_rn(sacc, Rp[r]);
-    }
-    // x = tstar * 2^-(S-1); the mantissa of t_j at exponent E is rint(x_j * 2^(S-1-E)).
-    // fits() is monotone in E, so the smallest fitting E is found by stepping
-    // from an estimate.
-    unsigned long long xm = 0;
-#pragma unroll
-    for (int j = 0; j < K; ++j) xm = max(xm, mag_bits(x[j]));
-    int E = xm ? ((int)(xm >> 52) - 1023) + (S - 1) - 2 : -8;
-    E = E < -8 ? -8 : (E > 7 ? 7 : E);
-    while (E > -8 && fits<K>(x, S - 1 - (E - 1))) --E;
-    while (E < 7 && !fits<K>(x, S - 1 - E)) ++E;
-    int t[K];
-#pragma unroll
-    for (int j = 0; j < K; ++j) {
-      double m = rint(scale2(x[j], S - 1 - E));
-      m = m < -8.0 ? -8.0 : (m > 7.0 ? 7.0 : m);
-      t[j] = (int)m;
-    }
-    // Quantized squared error, summed in i order.
-    double err = 0.0;
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      int Ri = 0;
-#pragma unroll
-      for (int j = 0; j < K; ++j) Ri += u[i][j] * t[j];
-      const double d = __dsub_rn(w[i], exact_d(Ri < 0, (unsigned long long)(Ri < 0 ? -Ri : Ri), 1 - S + E));
-      err = __dadd_rn(err, __dmul_rn(d, d));
-    }
+    seed_matrix<K>(S, Q, u);
+    SeedFactor<K> F;
+    factor_seed<K>(S, u, F);
+    if (F.singular) continue;
+    int E, t[6];
+    const double err = solve_block<K>(S, Q, u, F, B, wf, E, t);
     if (err < best) {
       best = err;
       bseed = s;
       bE = E;
 #pragma unroll
-      for (int j = 0; j < K; ++j) bt[j] = t[j];
+      for (int j = 0; j < 6; ++j) bt[j] = t[j];
     }
   }
 }
@@ -268,41 +100,13 @@ __device__ __forceinline__ void warp_best(double &best, uint32_t &bseed, int &bE
   }
 }
 
-struct EncodeOut {
-  uint32_t *seed;
-  int8_t *E;
-  int8_t *t;   // 6 per block
-  double *err;
-};
-
-__device__ __forceinline__ void write_out(const EncodeOut &o, int64_t blk, double best, uint32_t bseed,
-                                          int bE, const int (&bt)[6], int K) {
-  o.seed[blk] = bseed;
-  o.E[blk] = (int8_t)bE;
-  for (int j = 0; j < 6; ++j) o.t[blk * 6 + j] = (int8_t)(j < K ? bt[j] : 0);
-  if (o.err) o.err[blk] = best;
-}
-
 template <int K>
 __device__ __forceinline__ void encode_one(int S, const uint64_t *tab, const float (&w)[8], int lane,
                                            const EncodeOut &o, int64_t blk) {
   double best;
   uint32_t bseed;
   int bE, bt[6];
-  // Exponent spread of the block's weights (zeros do not constrain it).
-  int emin = 1 << 20, emax = -(1 << 20);
-#pragma unroll
-  for (int i = 0; i < 8; ++i) {
-    const unsigned int fb = __float_as_uint(w[i]);
-    if (fb & 0x7fffffffu) {
-      const int ef = (int)((fb >> 23) & 255u);
-      const int e = (ef ? ef : 1) - 150;
-      emin = min(emin, e);
-      emax = max(emax, e);
-    }
-  }
-  if (emax - emin <= 11) search_block<K, true>(S, tab, w, lane, best, bseed, bE, bt);
-  else search_block<K, false>(S, tab, w, lane, best, bseed, bE, bt);
+  search_block<K>(S, tab, w, lane, best, bseed, bE, bt);
   warp_best(best, bseed, bE, bt);
   if (lane == 0) write_out(o, blk, best, bseed, bE, bt, K);
 }
@@ -351,16 +155,7 @@ __global__ void __launch_bounds__(kEncWarps * 32) k_encode_layer(const __grid_co
     for (int j = 0; j < p.J - 1; ++j) bk[j] = __ldg(p.brk + r * (p.J - 1) + j);
     const int g = rung_of(bk, p.J, c);
     float wv[8];
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const int col = __ldg(p.perm + 8 * c + i);
-      // Outlier columns are stored in FP16 and overwrite the decode (Sec. 3.5):
-      // the search sees them as zero, so their spike does not leak into the
-      // block-mates.
-      bool outlier = false;
-      for (int o = 0; o < p.n_out; ++o) outlier |= (p.out_cols[o] == col);
-      wv[i] = outlier ? 0.f : __ldg(W + r * p.C + col);
-    }
+    gather_block(p, W, r, c, wv);
     encode_dispatch(rung_S(p.code[g]), rung_K(p.code[g]), tabs + (size_t)p.slot[g] * 512, wv, lane, o, blk);
   }
 }
@@ -428,6 +223,11 @@ seedq_status seedq_encode_blocks(int32_t S, int32_t k, const float *w, int64_t n
   if (nblocks < 0 || (nblocks > 0 && (!w || !seed || !E || !t))) return SEEDQ_ERR_INVALID_ARG;
   if (nblocks == 0) return SEEDQ_OK;
   EncodeOut o{seed, E, t, err};
+  if (screened(S, k, nblocks)) {
+    cudaError_t se;
+    if (screen_blocks(S, k, w, nblocks, o, (cudaStream_t)cuda_stream, &se))
+      return se == cudaSuccess ? SEEDQ_OK : cuda_fail(se);
+  }
   k_encode_list<<<grid_for(nblocks), kEncWarps * 32, 0, (cudaStream_t)cuda_stream>>>(
       S, k, seedq_lfsr_taps(S), w, nblocks, o);
   const cudaError_t e = cudaGetLastError();
@@ -439,6 +239,16 @@ seedq_status seedq_encode_layer(const seedq_layer *L, const float *W, uint32_t *
   if (!L || !W || !seed || !E || !t) return SEEDQ_ERR_INVALID_ARG;
   const int64_t total = L->args.R * (int64_t)L->args.nb;
   EncodeOut o{seed, E, t, err};
+  int maxS = 0, maxK = 0;
+  for (int j = 0; j < L->args.J; ++j) {
+    maxS = L->S[j] > maxS ? L->S[j] : maxS;
+    maxK = L->k[j] > maxK ? L->k[j] : maxK;
+  }
+  if (screened(maxS, maxK, total)) {
+    cudaError_t se;
+    if (screen_layer(L, W, o, (cudaStream_t)cuda_stream, &se))
+      return se == cudaSuccess ? SEEDQ_OK : cuda_fail(se);
+  }
   const size_t smem = sizeof(uint64_t) * 512 * (size_t)L->args.nslots;
   k_encode_layer<<<grid_for(total), kEncWarps * 32, smem, (cudaStream_t)cuda_stream>>>(L->args, W, o);
   const cudaError_t e = cudaGetLastError();

@@ -562,6 +562,18 @@ __device__ __forceinline__ DivRecip div_recip(double b) {
   return r;
 }
 
+// The same from a stored reciprocal estimate.
+__device__ __forceinline__ DivRecip div_recip_from(double b, uint64_t inv) {
+  const uint64_t bb = (uint64_t)__double_as_longlong(b);
+  DivRecip r;
+  r.b = b;
+  r.sign = bb >> 63;
+  r.e = (int)((bb >> 52) & 2047) - 1023;
+  r.d = (bb & ((1ull << 52) - 1)) | (1ull << 52);
+  r.inv = inv;
+  return r;
+}
+
 __device__ __forceinline__ double div_rn(double a, const DivRecip &R) {
   const uint64_t ab = (uint64_t)__double_as_longlong(a);
   const uint64_t sign = (ab >> 63) ^ R.sign;
@@ -582,22 +594,16 @@ __device__ __forceinline__ double div_rn(double a, const DivRecip &R) {
   mul128(q, R.d, phi, plo);
   long long rhi = (long long)(nhi - phi - (nlo < plo ? 1ull : 0ull));
   uint64_t rlo = nlo - plo;
-#pragma unroll
-  for (int k = 0; k < 3; ++k) {
-    if (rhi < 0) {  // remainder negative: q too large
-      --q;
-      const uint64_t t = rlo + R.d;
-      rhi += (t < rlo) ? 1 : 0;
-      rlo = t;
-    }
+  while (rhi < 0) {  // remainder negative: q too large
+    --q;
+    const uint64_t t = rlo + R.d;
+    rhi += (t < rlo) ? 1 : 0;
+    rlo = t;
   }
-#pragma unroll
-  for (int k = 0; k < 3; ++k) {
-    if (rhi > 0 || rlo >= R.d) {  // remainder >= d: q too small
-      ++q;
-      rhi -= (rlo < R.d) ? 1 : 0;
-      rlo -= R.d;
-    }
+  while (rhi > 0 || rlo >= R.d) {  // remainder >= d: q too small
+    ++q;
+    rhi -= (rlo < R.d) ? 1 : 0;
+    rlo -= R.d;
   }
   if (2 * rlo > R.d) ++q;  // round to nearest (no ties)
   if (q == (1ull << 53)) {
