@@ -1,4 +1,11 @@
 // Alg. 2 in full: materialize W_hat (rows of it) in the original column order.
+//
+// Two kernels.  k_decode_tile builds whole rows in shared memory, where the
+// scatter through the inverse permutation costs bank conflicts, and writes
+// them out as one contiguous bulk copy; it takes every tensor whose row fits.
+// k_decode scatters straight to memory, four bytes to a 32-byte sector: it is
+// left with rows too long for shared memory and outputs that are not 16-byte
+// aligned.
 #include <cuda_fp16.h>
 
 #include "seedq_internal.cuh"
@@ -17,7 +24,7 @@ __device__ __forceinline__ void decode_block(const LayerArgs &p, int S, uint64_t
   for (int i = 0; i < 8; ++i) Wrow[__ldg(p.perm + 8 * c + i)] = I[i] * scale;  // exact
 }
 
-// One thread per block; reads l(g_b) bits at the block's offset (row offset +
+// One thread per block, straight to memory; reads l(g_b) bits at the block's offset (row offset +
 // closed form over the row's rung breakpoints), writes 8 weights through the
 // inverse permutation (the scatter step of Alg. 2).
 __global__ void __launch_bounds__(256) k_decode(const __grid_constant__ LayerArgs p, int64_t row0, int64_t nrows, float *W) {
@@ -66,6 +73,313 @@ __global__ void k_outliers(const __grid_constant__ LayerArgs p, int64_t row0, in
   }
 }
 
+// ------------------------------------------------------------ whole rows
+//
+// One CTA per SM takes tiles of consecutive rows (contiguous in W and in the
+// stream).  Its last warp copies the tiles' stream bytes in a few tiles ahead
+// (cp.async.bulk on an mbarrier, with the rows' records) and, when the decoding
+// warps have all arrived on a second mbarrier, writes the finished tile out
+// with one bulk copy and hands the buffer back on a third.  The decoding warps
+// so wait neither for memory nor for the slowest of them.  A warp decodes 32
+// neighbouring blocks of a row at a time and scatters their weights through
+// the permutation (16-bit copy in shared memory).  Outlier columns are
+// overwritten in the buffer by the thread that wrote them.
+//
+// Bound by issue (63% of cycles) and the shared-memory pipe (61%: the scatter's
+// eight random words a block, two table lookups, the rung's constants), ahead
+// of the 4 bytes a weight written.  Measured against k_decode on one GB300:
+// 4096 x 11008 with a row factor and four outlier columns 286 -> 72 us (2.8
+// TB/s of weights and stream), 4096 x 4096 94 -> 32, 1024 x 1024 14 -> 10,
+// 512 x 20000 64 -> 29, 33 x 128 10 -> 7; no size in its range was slower.
+// On the way: two 512-thread CTAs per SM with barriers around each tile 88 us;
+// the moving warp instead of barriers 80; stream and permutation in shared
+// memory 80; chunks dealt from where the last tile ended 72 (the warps with
+// the odd chunk of every row had been the slow ones).  960 decoding threads
+// (64 registers, spills) 76, 608 72.5.
+constexpr int kDecThreads = 736;                // decoding threads (80 registers); one more warp moves data
+constexpr int kDecWarps = kDecThreads / 32;
+constexpr int kDecRows = 32;                    // rows per tile at most
+constexpr int kDecStages = 4;                   // tiles whose stream bytes are in flight or in use
+constexpr int kDecSmemMax = 227 * 1024;
+
+struct __align__(16) DecRow {
+  int32_t bk[kMaxJ - 1];    // breakpoints, kMaxCols past J - 1
+  int32_t base[kMaxJ];      // block c of rung g starts at staged bit base[g] + L[g] c
+  int32_t end;              // staged bit of the next row
+  uint32_t words;           // staged words of the tile
+  uint64_t word0;           // the tile's first staged word in the stream
+};
+
+struct DecFixed {
+  uint64_t tabs[kTableSlots * 512];
+  uint4 rdn[kMaxJ * RungDn<2>::kEntry];
+  uint4 rung[kMaxJ];                 // L, K, first table entry
+  DecRow row[kDecStages][kDecRows];
+  uint32_t outl[kMaxCols / 8 / 32];  // nonzero: the 32 blocks hold an outlier column
+  uint64_t ready[kDecStages];        // mbarriers: a stage's stream bytes and records are in place
+  uint64_t full[2];                  // per buffer: every decoding warp is through with the tile
+  uint64_t free_[2];                 // per buffer: its tile has been read for the copy out
+};
+
+__device__ __forceinline__ void mbar_init(uint64_t *b, uint32_t count) {
+  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"((uint32_t)__cvta_generic_to_shared(b)), "r"(count) : "memory");
+}
+__device__ __forceinline__ void mbar_arrive(uint64_t *b) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"((uint32_t)__cvta_generic_to_shared(b)) : "memory");
+}
+// Waits for the phase of the given parity; false after about a second.
+__device__ __forceinline__ bool mbar_wait(uint64_t *b, uint32_t parity) {
+  for (int i = 0; i < (1 << 20); ++i) {
+    uint32_t done;
+    asm volatile(
+        "{\n\t.reg .pred q;\n\tmbarrier.try_wait.parity.shared::cta.b64 q, [%1], %2, 1000;\n\tselp.u32 %0, 1, 0, q;\n\t}"
+        : "=r"(done) : "r"((uint32_t)__cvta_generic_to_shared(b)), "r"(parity) : "memory");
+    if (done) return true;
+  }
+  return false;
+}
+
+// Rung records of the tile's rows (one lane per row).  Bits relative to the
+// staged bytes fit 32 bits: a tile has at most kDecRows * kMaxCols / 8 blocks.
+__device__ __forceinline__ void dec_rows(const LayerArgs &p, int64_t r0, int nr, uint64_t word0, uint32_t words,
+                                         DecRow *rows) {
+  const int l = threadIdx.x & 31;
+  if (l >= nr) return;
+  // Rung g spans blocks [bk[g-1], bk[g]).
+  DecRow &R = rows[l];
+  const int64_t r = r0 + l;
+  int32_t base = (int32_t)(__ldg(p.row_off + r) - word0 * 32);
+  R.base[0] = base;
+  R.end = (int32_t)(__ldg(p.row_off + r + 1) - word0 * 32);
+  R.word0 = word0;
+  R.words = words;
+#pragma unroll
+  for (int j = 0; j < kMaxJ - 1; ++j) {
+    const int bk = j < p.J - 1 ? __ldg(p.brk + r * (p.J - 1) + j) : kMaxCols;
+    R.bk[j] = bk;
+    base -= p.dL[j] * bk;
+    R.base[j + 1] = base;
+  }
+}
+
+template <int K>
+__device__ __forceinline__ void decode_dn(uint32_t lo, uint32_t hi, const uint64_t *tab, const uint4 *rent, float (&w)[8]) {
+  const RungDn<K> rc(rent);
+  uint64_t I2[4];
+  float scale;
+  reconstruct_dn<K>(lo, hi, tab, rc, I2, scale);
+  // Powers of two: exact.
+  const uint64_t s2 = f2_pack(scale, scale * (1.0f / (float)(1 << RungDn<K>::Ko)));
+#pragma unroll
+  for (int p = 0; p < 4; ++p) {
+    const float2 v = f2_unpack(f2_mul(I2[p], s2));
+    w[2 * p] = v.x;
+    w[2 * p + 1] = v.y;
+  }
+}
+
+// Shared memory behind the fixed part: the permutation, then nbuf buffers of
+// trows rows of weights and kDecStages of their stream bytes.
+struct DecLayout {
+  int trows, nbuf;
+  uint32_t buf, buf_bytes, str, str_bytes, total;
+};
+constexpr uint32_t kDecFixed = (sizeof(DecFixed) + 127) / 128 * 128;
+
+__host__ __device__ inline uint32_t dec_stream_bytes(int trows, int nb) {
+  // Blocks of at most 44 bits, the last one's read-ahead and the alignment.
+  return (uint32_t)(((int64_t)trows * nb * 44 / 8 + 12 + 32 + 127) / 128 * 128);
+}
+
+static DecLayout dec_layout(int64_t C, int trows, int nbuf) {
+  DecLayout l;
+  l.trows = trows;
+  l.nbuf = nbuf;
+  l.buf_bytes = (uint32_t)((trows * C * 4 + 127) / 128 * 128);
+  l.str_bytes = dec_stream_bytes(trows, (int)(C / 8));
+  l.buf = (uint32_t)((kDecFixed + 2 * C + 127) / 128 * 128);
+  l.str = l.buf + nbuf * l.buf_bytes;
+  l.total = l.str + kDecStages * l.str_bytes;
+  return l;
+}
+
+__global__ void __launch_bounds__(kDecThreads + 32, 1)
+    k_decode_tile(const __grid_constant__ LayerArgs p, int64_t row0, int64_t nrows, float *W, const DecLayout lay) {
+  extern __shared__ __align__(128) uint8_t smem[];
+  DecFixed &F = *reinterpret_cast<DecFixed *>(smem);
+  uint16_t *perm = reinterpret_cast<uint16_t *>(smem + kDecFixed);
+  const int t = threadIdx.x, trows = lay.trows, nbuf = lay.nbuf;
+  for (int i = t; i < (int)p.C; i += kDecThreads + 32) perm[i] = (uint16_t)__ldg(p.perm + i);
+  {
+    const uint4 *src = reinterpret_cast<const uint4 *>(p.tables);
+    uint4 *dst = reinterpret_cast<uint4 *>(F.tabs);
+    for (int i = t; i < kTableSlots * 256; i += kDecThreads + 32) dst[i] = __ldg(src + i);
+    for (int i = t; i < kMaxCols / 8 / 32; i += kDecThreads + 32) F.outl[i] = 0u;
+    if (t < p.J) F.rung[t] = make_uint4(p.L[t], rung_K(p.code[t]), p.slot[t] * 512, 0u);
+  }
+  store_rung_entries(p, p.zero, F.rdn);
+  if (t == 0) {
+    for (int b = 0; b < kDecStages; ++b) mbar_init(F.ready + b, 1);
+    for (int b = 0; b < 2; ++b) {
+      mbar_init(F.full + b, kDecWarps);
+      mbar_init(F.free_ + b, 1);
+    }
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  __syncthreads();
+  if (t < p.n_out) {
+    const int c = __ldg(p.invperm + p.out_cols[t]) >> 3;
+    F.outl[c >> 5] = 1u;
+  }
+  __syncthreads();
+  const int64_t tiles = (nrows + trows - 1) / trows;
+  const int C = (int)p.C;
+  if (t >= kDecThreads) {
+    // The moving warp.
+    auto stage = [&](int64_t tile, int b) {
+      if (tile >= tiles) return;
+      const int nr = (int)min((int64_t)trows, nrows - tile * trows);
+      const int64_t r0 = row0 + tile * trows;
+      // The tile's stream bytes: whole 16-byte pieces, cut where the readable
+      // buffer ends and at the stage's size.
+      const uint64_t lo = (__ldg(p.row_off + r0) >> 3) & ~(uint64_t)15;
+      uint64_t hi = (((__ldg(p.row_off + r0 + nr) + 96 + 7) >> 3) + 15) & ~(uint64_t)15;
+      hi = min(hi, min(p.stream_words * 4, lo + lay.str_bytes) & ~(uint64_t)15);
+      const uint32_t bytes = hi > lo ? (uint32_t)(hi - lo) : 0u;
+      dec_rows(p, r0, nr, lo >> 2, bytes >> 2, F.row[b]);
+      __syncwarp();
+      if (t == kDecThreads) {
+        const uint32_t bar = (uint32_t)__cvta_generic_to_shared(F.ready + b);
+        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
+        if (bytes)
+          asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+                           (uint32_t)__cvta_generic_to_shared(smem + lay.str + b * lay.str_bytes)),
+                       "l"(reinterpret_cast<const uint8_t *>(p.stream) + lo), "r"(bytes), "r"(bar)
+                       : "memory");
+      }
+      __syncwarp();
+    };
+    for (int b = 0; b < kDecStages; ++b) stage(blockIdx.x + (int64_t)b * gridDim.x, b);
+    uint32_t b = 0, ph = 0, sb = 0;
+    for (int64_t tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
+      if (!mbar_wait(F.full + b, ph)) {
+        atomicOr(p.flags, 1u);
+        break;
+      }
+      if (t == kDecThreads) {
+        const int64_t n0 = tile * trows;
+        asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(W + n0 * p.C),
+                     "r"((uint32_t)__cvta_generic_to_shared(smem + lay.buf + b * lay.buf_bytes)),
+                     "r"((uint32_t)(min((int64_t)trows, nrows - n0) * C * 4))
+                     : "memory");
+        asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+      }
+      stage(tile + (int64_t)kDecStages * gridDim.x, sb);
+      if (t == kDecThreads) {
+        asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+        mbar_arrive(F.free_ + b);
+      }
+      sb = sb + 1 == kDecStages ? 0 : sb + 1;
+      if (++b == (uint32_t)nbuf) {
+        b = 0;
+        ph ^= 1;
+      }
+    }
+    if (t == kDecThreads) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
+    return;
+  }
+  uint32_t b = 0, ph = 0, sb = 0, sph = 0;
+  int chunk = t >> 5;  // the warp's first chunk of the tile
+  for (int64_t tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
+    const int64_t i0 = tile * trows;
+    const int nr = (int)min((int64_t)trows, nrows - i0);
+    float *buf = reinterpret_cast<float *>(smem + lay.buf + b * lay.buf_bytes);
+    const uint32_t *str = reinterpret_cast<const uint32_t *>(smem + lay.str + sb * lay.str_bytes);
+    const DecRow *rows = F.row[sb];
+    // (A buffer's first use finds the phase before its first release complete.)
+    if (!mbar_wait(F.ready + sb, sph) || !mbar_wait(F.free_ + b, ph ^ 1)) {
+      atomicOr(p.flags, 1u);
+      return;
+    }
+    // The tile's rows in chunks of 32 columns, dealt to the warps round-robin
+    // from where the last tile's deal ended, so that no warp draws more.
+    const int lane = t & 31, cpr = (p.nb + 31) / 32, chunks = nr * cpr;
+    for (int k = chunk; k < chunks; k += kDecWarps) {
+      const int i = k / cpr, k0 = k - i * cpr, c = k0 * 32 + lane;
+      const DecRow &R = rows[i];
+      // The chunk's first rung by one compare per lane; a lane past a
+      // breakpoint inside the chunk moves on from there.
+      int g = __popc(__ballot_sync(0xffffffffu, lane < kMaxJ - 1 && k0 * 32 >= R.bk[lane & 7]));
+      while (c >= R.bk[g & 7] && g < kMaxJ - 1) ++g;
+      const uint4 rg = F.rung[g];
+      const int off = R.base[g] + (int)rg.x * c;
+      const uint32_t at = (uint32_t)off >> 5;
+      const bool ok = c < p.nb;
+      // As k_decode: the plan and the bound buffer must agree.
+      if (c == p.nb - 1 && off + (int)rg.x != R.end) atomicOr(p.flags, 1u);
+      if (!ok) continue;
+      const uint4 pc = *reinterpret_cast<const uint4 *>(perm + 8 * c);
+      const uint32_t col[8] = {pc.x & 0xffffu, pc.x >> 16, pc.y & 0xffffu, pc.y >> 16,
+                               pc.z & 0xffffu, pc.z >> 16, pc.w & 0xffffu, pc.w >> 16};
+      float w[8];
+      uint32_t w0, w1, w2;
+      bool readable = true;
+      if (at + 3 <= R.words) {
+        w0 = str[at];
+        w1 = str[at + 1];
+        w2 = str[at + 2];
+      } else {  // the last words of a buffer that is cut short or not a multiple of 16 bytes
+        const uint64_t wi = R.word0 + at;
+        readable = wi + 3 <= p.stream_words;
+        w0 = readable ? __ldg(p.stream + wi) : 0u;
+        w1 = readable ? __ldg(p.stream + wi + 1) : 0u;
+        w2 = readable ? __ldg(p.stream + wi + 2) : 0u;
+      }
+      const uint32_t lo = __funnelshift_r(w0, w1, (uint32_t)off), hi = __funnelshift_r(w1, w2, (uint32_t)off);
+      const uint64_t *tab = F.tabs + rg.z;
+      const uint4 *rent = F.rdn + g * RungDn<2>::kEntry;
+      switch (rg.y) {
+        case 2: decode_dn<2>(lo, hi, tab, rent, w); break;
+        case 3: decode_dn<3>(lo, hi, tab, rent, w); break;
+        case 4: decode_dn<4>(lo, hi, tab, rent, w); break;
+        case 5: decode_dn<5>(lo, hi, tab, rent, w); break;
+        default: decode_dn<6>(lo, hi, tab, rent, w); break;
+      }
+      float *brow = buf + i * C;
+      if (!readable) {
+        atomicOr(p.flags, 1u);
+        const float *old = W + (i0 + i) * p.C;  // a block that cannot be read keeps what W holds
+#pragma unroll
+        for (int e = 0; e < 8; ++e) w[e] = old[col[e]];
+      }
+#pragma unroll
+      for (int e = 0; e < 8; ++e) brow[col[e]] = w[e];
+      if (F.outl[k0]) {
+        const int first = c * 8;
+        for (int o = 0; o < p.n_out; ++o) {
+          const int at_o = __ldg(p.invperm + p.out_cols[o]) - first;
+          if (at_o >= 0 && at_o < 8)
+            brow[p.out_cols[o]] = __half2float(__ushort_as_half(__ldg(p.out_vals + (row0 + i0 + i) * p.n_out + o)));
+        }
+      }
+    }
+    chunk -= chunks % kDecWarps;
+    if (chunk < 0) chunk += kDecWarps;
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    __syncwarp();
+    if ((t & 31) == 0) mbar_arrive(F.full + b);
+    if (++sb == kDecStages) {
+      sb = 0;
+      sph ^= 1;
+    }
+    if (++b == (uint32_t)nbuf) {
+      b = 0;
+      ph ^= 1;
+    }
+  }
+}
+static_assert(kDecRows <= 32, "one lane of the storing warp per row record");
+
 }  // namespace seedq
 
 using namespace seedq;
@@ -81,6 +395,28 @@ seedq_status seedq_decode_rows(const seedq_layer *L, int64_t row0, int64_t nrows
   int dev = 0, sms = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  const int64_t C = L->args.C;
+  DecLayout lay = dec_layout(C, 1, 2);
+  if (lay.total > (uint32_t)kDecSmemMax) lay = dec_layout(C, 1, 1);
+  if (((uintptr_t)W & 15u) == 0 && lay.total <= (uint32_t)kDecSmemMax) {
+    // Rows per tile: as many as fit twice, fewer when each SM would get less
+    // than four tiles, but at least a chunk for every decoding warp while that
+    // leaves each SM a tile.
+    if (lay.nbuf == 2) {
+      const int64_t cpr = (L->args.nb + 31) / 32, fill = kDecWarps / cpr, each = (nrows + sms - 1) / sms;
+      int64_t rows = nrows / (4 * sms), least = fill < each ? fill : each;
+      rows = rows < least ? least : rows;
+      rows = rows > kDecRows ? kDecRows : rows;
+      while (rows > 1 && dec_layout(C, (int)rows, 2).total > (uint32_t)kDecSmemMax) --rows;
+      if (rows > 1) lay = dec_layout(C, (int)rows, 2);
+    }
+    const int64_t tiles = (nrows + lay.trows - 1) / lay.trows;
+    // Per call: the attribute belongs to the current device.
+    SEEDQ_CUDA(cudaFuncSetAttribute(k_decode_tile, cudaFuncAttributeMaxDynamicSharedMemorySize, kDecSmemMax));
+    k_decode_tile<<<(int)(tiles < sms ? tiles : sms), kDecThreads + 32, lay.total, st>>>(L->args, row0, nrows, W, lay);
+    SEEDQ_CUDA(cudaGetLastError());
+    return SEEDQ_OK;
+  }
   const int64_t blocks = nrows * (int64_t)L->args.nb;
   const int64_t want = (blocks + 255) / 256;
   const int grid = (int)(want < (int64_t)sms * 16 ? want : (int64_t)sms * 16);

@@ -193,22 +193,6 @@ __device__ __forceinline__ void dispatch_cols(int code, const uint4 *rent, const
   }
 }
 
-// The per-rung constants of RungDn for every rung of a tensor (thread j < J
-// writes rung j's entry).
-__device__ __forceinline__ void store_rung_entries(const LayerArgs &p, uint32_t z, uint4 *rdn) {
-  const int j = threadIdx.x;
-  if (j >= p.J) return;
-  const int code = p.code[j], S = rung_S(code);
-  uint4 *e = rdn + j * RungDn<2>::kEntry;
-  switch (rung_K(code)) {
-    case 2: RungDn<2>(S, z).store(e); break;
-    case 3: RungDn<3>(S, z).store(e); break;
-    case 4: RungDn<4>(S, z).store(e); break;
-    case 5: RungDn<5>(S, z).store(e); break;
-    default: RungDn<6>(S, z).store(e); break;
-  }
-}
-
 // Bits of the lane's row before blocks cs and ce.  Rung j spans blocks
 // [bk[j-1], bk[j]) and the breakpoints rise along the row, so the bits before
 // block x are L[0] x plus, for every breakpoint below x, the rate step dL[j]

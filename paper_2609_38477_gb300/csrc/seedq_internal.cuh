@@ -435,6 +435,22 @@ struct RungDn {
   }
 };
 
+// The per-rung constants of RungDn for every rung of a tensor (thread j < J
+// writes rung j's entry).
+__device__ __forceinline__ void store_rung_entries(const LayerArgs &p, uint32_t z, uint4 *rdn) {
+  const int j = threadIdx.x;
+  if (j >= p.J) return;
+  const int code = p.code[j], S = rung_S(code);
+  uint4 *e = rdn + j * RungDn<2>::kEntry;
+  switch (rung_K(code)) {
+    case 2: RungDn<2>(S, z).store(e); break;
+    case 3: RungDn<3>(S, z).store(e); break;
+    case 4: RungDn<4>(S, z).store(e); break;
+    case 5: RungDn<5>(S, z).store(e); break;
+    default: RungDn<6>(S, z).store(e); break;
+  }
+}
+
 // Bits [N, N + 32) of Q = (qhi:qlo), zero past bit 63 (0 <= N < 64).
 template <int N>
 __device__ __forceinline__ uint32_t qwin2(uint32_t qlo, uint32_t qhi) {
