@@ -121,21 +121,31 @@ __global__ void __launch_bounds__(kRankChunk / 2) k_chunk_sort(const RankJob<K> 
 
 template <typename K, bool kDesc>
 __global__ void __launch_bounds__(256) k_chunk_rank(const RankJob<K> *__restrict__ jobs, int nj) {
-  const RankJob<K> &J = jobs[rank_job(jobs, nj, blockIdx.x, false)];
+  // The chunks pass through shared memory: the binary searches' gathers were
+  // bound by the L1 pipe (35,584 keys of seven tensors: 72 -> 23 us).
+  __shared__ K sk[kRankChunk];
+  __shared__ int32_t si[kRankChunk];
+  const RankJob<K> J = jobs[rank_job(jobs, nj, blockIdx.x, false)];
   const int i = (blockIdx.x - J.rblk0) * 256 + threadIdx.x;
-  if (i >= J.n) return;
-  const K ki = J.key[i];
+  const K ki = i < J.n ? J.key[i] : K(0);
   int rank = 0;
   for (int c0 = 0; c0 < J.n; c0 += kRankChunk) {
-    int lo = 0, hi = min(kRankChunk, J.n - c0);
+    const int n = min(kRankChunk, J.n - c0);
+    __syncthreads();
+    for (int t = threadIdx.x; t < n; t += 256) {
+      sk[t] = J.skey[c0 + t];
+      si[t] = J.sidx[c0 + t];
+    }
+    __syncthreads();
+    int lo = 0, hi = n;
     while (lo < hi) {
       const int mid = (lo + hi) >> 1;
-      if (rank_less<K, kDesc>(J.skey[c0 + mid], J.sidx[c0 + mid], ki, i)) lo = mid + 1;
+      if (rank_less<K, kDesc>(sk[mid], si[mid], ki, i)) lo = mid + 1;
       else hi = mid;
     }
     rank += lo;
   }
-  J.out[rank] = i;
+  if (i < J.n) J.out[rank] = i;
 }
 
 // Launches the two kernels over nj jobs whose descriptors (with block numbers
@@ -187,22 +197,83 @@ __global__ void k_invperm(const int32_t *__restrict__ perm, int C, int32_t *__re
   if (i < C) inv[perm[i]] = i;
 }
 
+// Whether every sum of n values with these exponents is exact in fp64: all are
+// multiples of 2^(lsb) and below 2^(top), so any partial sum needs at most
+// top + log2(n) - lsb bits.  Then the order does not matter.
+__device__ __forceinline__ bool sum_is_exact(int lsb, int top, int64_t n) {
+  return top + (64 - __clzll((long long)n)) - lsb <= 53;
+}
+
+// Lowest bit and power-of-two bound over the nonzero values of v (a block-wide
+// reduction; lsb > top when all are zero).
+__device__ void exponent_range(const float *__restrict__ v, int64_t n, int &lsb, int &top) {
+  __shared__ int s_lsb, s_top;
+  if (threadIdx.x == 0) {
+    s_lsb = 1 << 20;
+    s_top = -(1 << 20);
+  }
+  __syncthreads();
+  int l = 1 << 20, t = -(1 << 20);
+  for (int64_t i = threadIdx.x; i < n; i += blockDim.x) {
+    const uint32_t b = __float_as_uint(v[i]) & 0x7fffffffu;
+    if (!b) continue;
+    const int e = max((int)(b >> 23), 1);
+    l = min(l, e - 150);
+    t = max(t, e - 126);
+  }
+  l = __reduce_min_sync(0xffffffffu, l);
+  t = __reduce_max_sync(0xffffffffu, t);
+  if ((threadIdx.x & 31) == 0) {
+    atomicMin(&s_lsb, l);
+    atomicMax(&s_top, t);
+  }
+  __syncthreads();
+  lsb = s_lsb;
+  top = s_top;
+  __syncthreads();
+}
+
+// Sum of the threads' values (any order; for sums known to be exact).
+__device__ double block_total(double x) {
+  __shared__ double part[32];
+  for (int o = 16; o > 0; o >>= 1) x = __dadd_rn(x, __shfl_xor_sync(0xffffffffu, x, o));
+  __syncthreads();
+  if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = x;
+  __syncthreads();
+  double s = 0.0;
+  for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s = __dadd_rn(s, part[w]);
+  return s;
+}
+
 // Block means of the permuted a, summed in channel order, and their unit-mean
 // normalization summed in ascending block order (Eq. imp; App. A.7 fixed order).
-// One thread block per tensor.
+// One thread block per tensor.  Where every partial sum is exact, which the
+// values' exponents tell, the sum over blocks is taken in parallel: the same
+// double without a chain of nb additions in one thread (nb = 1376: 16 us).
 __device__ __forceinline__ void abar_block(const float *__restrict__ a, const int32_t *__restrict__ perm,
                                            int nb, double *__restrict__ abar) {
   __shared__ double mean;
+  int lsb, top;
+  exponent_range(a, (int64_t)nb * 8, lsb, top);
+  double local = 0.0;
   for (int c = threadIdx.x; c < nb; c += blockDim.x) {
     double s = 0.0;
     for (int i = 0; i < 8; ++i) s = __dadd_rn(s, (double)a[perm[8 * c + i]]);
-    abar[c] = __ddiv_rn(s, 8.0);
+    const double v = __ddiv_rn(s, 8.0);
+    abar[c] = v;
+    local = __dadd_rn(local, v);
   }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double s = 0.0;
-    for (int c = 0; c < nb; ++c) s = __dadd_rn(s, abar[c]);
-    mean = __ddiv_rn(s, (double)nb);
+  // (The means are multiples of 2^(lsb - 3) and there are n / 8 of them.)
+  if (sum_is_exact(lsb, top, (int64_t)nb * 8)) {
+    const double s = block_total(local);
+    if (threadIdx.x == 0) mean = __ddiv_rn(s, (double)nb);
+  } else {
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      double s = 0.0;
+      for (int c = 0; c < nb; ++c) s = __dadd_rn(s, abar[c]);
+      mean = __ddiv_rn(s, (double)nb);
+    }
   }
   __syncthreads();
   for (int c = threadIdx.x; c < nb; c += blockDim.x) abar[c] = __ddiv_rn(abar[c], mean);
@@ -213,23 +284,43 @@ __global__ void k_abar(const float *__restrict__ a, const int32_t *__restrict__ 
   abar_block(a, perm, nb, abar);
 }
 
-// Row factor normalized to unit mean, summed in ascending row order.
+// Row factor normalized to unit mean, summed in ascending row order (in
+// parallel where exact, as above).
+// inv (optional): 1 / rho, slightly low (see first_blocks).
+constexpr double kSlightlyLow = 1.0 - 0x1p-48;
+
 __device__ __forceinline__ void rho_block(const float *__restrict__ rho_in, int64_t R,
-                                          double *__restrict__ rho) {
+                                          double *__restrict__ rho, double *__restrict__ inv) {
   __shared__ double mean;
-  if (threadIdx.x == 0) {
+  if (!rho_in) {
+    for (int64_t r = threadIdx.x; r < R; r += blockDim.x) {
+      rho[r] = 1.0;
+      if (inv) inv[r] = kSlightlyLow;
+    }
+    return;
+  }
+  int lsb, top;
+  exponent_range(rho_in, R, lsb, top);
+  if (sum_is_exact(lsb, top, R)) {
+    double local = 0.0;
+    for (int64_t r = threadIdx.x; r < R; r += blockDim.x) local = __dadd_rn(local, (double)rho_in[r]);
+    const double s = block_total(local);
+    if (threadIdx.x == 0) mean = __ddiv_rn(s, (double)R);
+  } else if (threadIdx.x == 0) {
     double s = 0.0;
-    if (rho_in)
-      for (int64_t r = 0; r < R; ++r) s = __dadd_rn(s, (double)rho_in[r]);
+    for (int64_t r = 0; r < R; ++r) s = __dadd_rn(s, (double)rho_in[r]);
     mean = __ddiv_rn(s, (double)R);
   }
   __syncthreads();
-  for (int64_t r = threadIdx.x; r < R; r += blockDim.x)
-    rho[r] = rho_in ? __ddiv_rn((double)rho_in[r], mean) : 1.0;
+  for (int64_t r = threadIdx.x; r < R; r += blockDim.x) {
+    const double v = __ddiv_rn((double)rho_in[r], mean);
+    rho[r] = v;
+    if (inv) inv[r] = __ddiv_rn(1.0, v) * kSlightlyLow;
+  }
 }
 
 __global__ void k_rho(const float *__restrict__ rho_in, int64_t R, double *__restrict__ rho) {
-  rho_block(rho_in, R, rho);
+  rho_block(rho_in, R, rho, nullptr);
 }
 
 // The same three steps for many tensors at once (the allocator's factors).
@@ -239,15 +330,15 @@ struct FacJob {
   int32_t *perm;        // C
   double *abar;         // C / 8
   double *rho;          // R
+  double *inv;          // R
   int64_t R;
   int32_t C;
 };
 
 __global__ void k_factors_multi(const FacJob *__restrict__ jobs) {
-  const FacJob &J = jobs[blockIdx.x];
-  abar_block(J.a, J.perm, J.C / 8, J.abar);
-  __syncthreads();
-  rho_block(J.rho_in, J.R, J.rho);
+  const FacJob J = jobs[blockIdx.x >> 1];
+  if (blockIdx.x & 1) rho_block(J.rho_in, J.R, J.rho, J.inv);
+  else abar_block(J.a, J.perm, J.C / 8, J.abar);
 }
 
 struct SchedArgs {
@@ -957,74 +1048,317 @@ extern "C" seedq_status seedq_row_plan_static(const double *abar, const double *
 
 // ------------------------------------------------------------ allocator
 // Alg. 1 over a set of tensors: every count is an integer summed with atomic
-// adds and every importance the same fp64 product as the plan's, so the
-// bisections take the same steps on any device and agree with a sequential
-// evaluation.
+// adds and every importance the same fp64 product as the plan's.  Both
+// searches (the floor's order statistic and the multiplier) look for the one
+// place where a monotone integer count crosses a target, so any way of halving
+// the interval ends there: the result agrees with a sequential bisection.
+//
+// The searches run on the device, round after round without a host read: a
+// round evaluates `probes` points of the interval at once and its last block
+// narrows the interval for the next.  With few rows a round is bound by its
+// launch, so it takes up to 31 points (14 rounds instead of 63 steps); with many
+// by the binary searches, so it takes one.
 namespace seedq {
 namespace {
 
 struct AllocTensor {
   const double *abar;  // nb unit-mean block means (ascending)
   const double *rho;   // rows unit-mean row factors
+  const double *inv;   // and their reciprocals, slightly low
   int64_t R;           // rows of the tensor
-  int64_t row0;        // first evaluated row in the launch's row space
+  int32_t blk0;        // first block of the tensor in a launch (256 evaluated rows a block)
   int32_t nrows;       // evaluated rows (1 when rho is 1 on every row)
   int32_t nb;
 };
 
-enum AllocMode { kCountLE = 0, kBits = 1, kVmin = 2, kTied = 3 };
+constexpr int kMaxProbes = 31;
+
+struct AllocState {
+  // Bit patterns of positive doubles.  Floor: the answer lies in [lo, hi].
+  // Multiplier: bits(lo) > budget >= bits(hi).
+  long long lo[2], hi[2];
+  unsigned long long cnt[kMaxProbes];  // the round's counts (0 between rounds)
+  unsigned long long vmin[kMaxJ];      // bit patterns: smallest importance at or above th_lo[j]
+  unsigned int arrive;                 // blocks finished (0 between launches)
+  int jt, ngroups;                     // critical rung and how many qualified
+  double v;                            // its importance
+};
 
 struct AllocArgs {
   const AllocTensor *t;
   int32_t nt;
-  int64_t rows;        // evaluated rows over all tensors
-  int32_t mode, J;
+  int32_t J;
   int32_t L[kMaxJ];
-  double q, v;
-  double th[kMaxJ];
-  unsigned long long *total;      // kCountLE / kBits / kTied: one counter
-  unsigned long long *per_tensor; // kBits / kTied: nt counters
-  unsigned long long *vmin;       // kVmin: J - 1 bit patterns
+  double slopes[kMaxJ];
+  unsigned long long target;  // floor: the rank m; multiplier: the budget
+  AllocState *st;
+  unsigned long long *bits;   // nt: payload bits per tensor at the final thresholds
+  unsigned long long *tied;   // nt: blocks per tensor at the critical importance
 };
 
-__global__ void k_alloc_eval(const __grid_constant__ AllocArgs a) {
-  const int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  unsigned long long val = 0;
-  int ti = -1;
-  if (g < a.rows) {
-    int lo = 0, hi = a.nt - 1;
-    while (lo < hi) {
-      const int mid = (lo + hi + 1) >> 1;
-      if (a.t[mid].row0 <= g) lo = mid;
-      else hi = mid - 1;
+__device__ __forceinline__ int alloc_tensor(const AllocArgs &a) {
+  int lo = 0, hi = a.nt - 1;
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (a.t[mid].blk0 <= (int)blockIdx.x) lo = mid;
+    else hi = mid - 1;
+  }
+  return lo;
+}
+
+// High words of the block's tensor's means, in shared memory where a warp's
+// worth of rows will search them.
+__device__ __forceinline__ const uint32_t *stage_high_words(const AllocTensor &T, uint32_t *sh, int &stride) {
+  const uint32_t *hw = reinterpret_cast<const uint32_t *>(T.abar) + 1;
+  stride = 2;
+  if (T.nrows < 32) return hw;
+  for (int i = threadIdx.x; i < T.nb; i += blockDim.x) sh[i] = __ldg(hw + 2 * i);
+  __syncthreads();
+  stride = 1;
+  return sh;
+}
+
+// first_block for n thresholds at once (strict: bit j set for importance >
+// thr[j] instead of >=), with the fp64 pipe, a sixty-fourth of the integer
+// pipes' rate, kept out of the searches: imp >= thr is abar rr >= thr (unless
+// the floor alone decides), which fails wherever abar's high word (hw; positive
+// and rising) is below that of thr / rr taken slightly low.  The searches run on high words, all in step
+// so that their loads overlap; the exact product decides from there on.
+template <int N>
+__device__ __forceinline__ void first_blocks(const double *abar, const uint32_t *hw, int stride, double rr,
+                                             double inv, double q, int nb, const double (&thr)[N], int n, uint32_t strict, int (&out)[N]) {
+  // Doubles here are never negative, so they compare as their bit patterns.
+  const long long qb = __double_as_longlong(q);
+  int lo[N], hi[N];
+  uint32_t key[N];
+#pragma unroll
+  for (int j = 0; j < N; ++j) {
+    const long long tb = __double_as_longlong(thr[j]);
+    const bool floor_passes = (strict >> j & 1u) ? qb > tb : qb >= tb;
+    lo[j] = 0;
+    hi[j] = (j < n && !floor_passes) ? nb : 0;
+    const uint32_t x = (uint32_t)__double2hiint(thr[j] * inv);
+    key[j] = x > 0x06000000u ? x : 0u;  // (products below 1e-279 lose their relative accuracy)
+  }
+  for (int s = nb; s > 0; s >>= 1) {
+#pragma unroll
+    for (int j = 0; j < N; ++j) {
+      const int mid = (lo[j] + hi[j]) >> 1;
+      const bool up = hw[min(mid, nb - 1) * stride] >= key[j], go = lo[j] < hi[j];
+      hi[j] = go && up ? mid : hi[j];
+      lo[j] = go && !up ? mid + 1 : lo[j];
     }
-    ti = lo;
-    const AllocTensor &T = a.t[ti];
-    const double rr = T.rho[g - T.row0];
-    const unsigned long long mult = T.nrows == 1 ? (unsigned long long)T.R : 1ull;
-    if (a.mode == kCountLE) {
-      val = (unsigned long long)first_block(T.abar, rr, -INFINITY, T.nb, a.v, true) * mult;
-    } else if (a.mode == kBits) {
-      unsigned long long rb = (unsigned long long)a.L[0] * (unsigned long long)T.nb;
-      for (int j = 0; j < a.J - 1; ++j) {
-        const int n_ge = T.nb - first_block(T.abar, rr, a.q, T.nb, a.th[j], false);
-        rb += (unsigned long long)(a.L[j + 1] - a.L[j]) * (unsigned long long)n_ge;
-      }
-      val = rb * mult;
-    } else if (a.mode == kTied) {
-      val = (unsigned long long)(first_block(T.abar, rr, a.q, T.nb, a.v, true) -
-                                 first_block(T.abar, rr, a.q, T.nb, a.v, false)) * mult;
+  }
+  // The first candidates' exact tests together; usually they pass.
+  long long at[N];
+#pragma unroll
+  for (int j = 0; j < N; ++j) at[j] = __double_as_longlong(__dmul_rn(abar[min(lo[j], nb - 1)], rr));
+#pragma unroll
+  for (int j = 0; j < N; ++j) {
+    const bool st = strict >> j & 1u;
+    const long long tb = __double_as_longlong(thr[j]);
+    out[j] = lo[j];
+    if (j >= n || lo[j] >= nb || (st ? qb > tb || at[j] > tb : qb >= tb || at[j] >= tb)) continue;
+    // A run of nearly equal means: one step, then a search.
+    int l = lo[j] + 1, h = nb;
+    bool first = true;
+    while (l < h) {
+      const int mid = first ? l : (l + h) >> 1;
+      first = false;
+      const long long v = __double_as_longlong(__dmul_rn(abar[mid], rr));
+      if (st ? v > tb : v >= tb) h = mid;
+      else l = mid + 1;
+    }
+    out[j] = l;
+  }
+}
+
+// Point i of n inside (lo, hi), in rising order.
+__device__ __forceinline__ long long probe_at(long long lo, long long hi, int i, int n) {
+  const unsigned long long d = (unsigned long long)(hi - lo), k = (unsigned long long)(i + 1);
+  const unsigned long long w = (unsigned long long)(n + 1);
+  return lo + (long long)(d / w * k + d % w * k / w);
+}
+
+// One round of a search (kFloor: count of importances <= v against the rank;
+// else payload bits at thresholds v / slope_j against the budget), blockIdx.y
+// the probe.
+template <bool kFloor>
+__global__ void __launch_bounds__(256) k_alloc_round(const __grid_constant__ AllocArgs a) {
+  // The block's rows and means do not change between rounds: fetched while the
+  // last round ends (programmatic dependent launch; its grid has to be
+  // complete before the state is read, and only then may the next one start).
+  __shared__ uint32_t s_hw[kMaxCols / 8];
+  const AllocTensor T = a.t[alloc_tensor(a)];
+  int stride;
+  const uint32_t *hw = stage_high_words(T, s_hw, stride);
+  const int row = (blockIdx.x - T.blk0) * blockDim.x + threadIdx.x;
+  const double rr = row < T.nrows ? T.rho[row] : 1.0, inv = row < T.nrows ? T.inv[row] : 1.0;
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;");
+  AllocState &S = *a.st;
+  const int which = kFloor ? 0 : 1, n = gridDim.y;
+  const long long lo = __ldcg(&S.lo[which]), hi = __ldcg(&S.hi[which]);
+  if (kFloor ? lo >= hi : hi - lo <= 1) return;  // done; the same in every block
+  const double v = __longlong_as_double(probe_at(lo, hi, blockIdx.y, n));
+  __shared__ double s_th[kMaxJ];
+  if (!kFloor) {
+    if (threadIdx.x < kMaxJ) s_th[threadIdx.x] = threadIdx.x < a.J - 1 ? __ddiv_rn(v, a.slopes[threadIdx.x]) : 0.0;
+    __syncthreads();
+  }
+  unsigned long long val = 0;
+  if (row < T.nrows) {
+    if (kFloor) {
+      const double th[1] = {v};
+      int c[1];
+      first_blocks<1>(T.abar, hw, stride, rr, inv, 0.0, T.nb, th, 1, 1u, c);
+      val = (unsigned long long)c[0];
     } else {
-      for (int j = 0; j < a.J - 1; ++j) {
-        const int c = first_block(T.abar, rr, a.q, T.nb, a.th[j], false);
-        if (c < T.nb) atomicMin(a.vmin + j, (unsigned long long)__double_as_longlong(imp_at(T.abar, rr, a.q, c)));
+      const double q = __longlong_as_double(__ldcg(&S.lo[0]));
+      double th[kMaxJ - 1];
+      int c[kMaxJ - 1];
+#pragma unroll
+      for (int j = 0; j < kMaxJ - 1; ++j) th[j] = s_th[j];
+      first_blocks<kMaxJ - 1>(T.abar, hw, stride, rr, inv, q, T.nb, th, a.J - 1, 0u, c);
+      val = (unsigned long long)a.L[0] * (unsigned long long)T.nb;
+#pragma unroll
+      for (int j = 0; j < kMaxJ - 1; ++j)
+        if (j < a.J - 1) val += (unsigned long long)(a.L[j + 1] - a.L[j]) * (unsigned long long)(T.nb - c[j]);
+    }
+    if (T.nrows == 1) val *= (unsigned long long)T.R;
+  }
+  for (int o = 16; o > 0; o >>= 1) val += __shfl_xor_sync(0xffffffffu, val, o);
+  __shared__ unsigned long long s_val[8];
+  __shared__ bool last;
+  if ((threadIdx.x & 31) == 0) s_val[threadIdx.x >> 5] = val;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < 8; ++w) val += s_val[w];
+    if (val) atomicAdd(S.cnt + blockIdx.y, val);
+    __threadfence();
+    last = atomicAdd(&S.arrive, 1u) == gridDim.x * gridDim.y - 1;
+  }
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  // Thread i (of the first warp) holds probe i's verdict; the crossing is the
+  // first probe on the far side.
+  if (threadIdx.x >= 32) return;
+  const int i = threadIdx.x;
+  const unsigned long long cnt = i < n ? __ldcg(S.cnt + i) : 0ull;
+  const unsigned far = __ballot_sync(0xffffffffu, i < n && (kFloor ? cnt >= a.target : cnt <= a.target));
+  if (i < n) S.cnt[i] = 0ull;
+  if (i == 0) {
+    const int k = far ? __ffs(far) - 1 : n;
+    if (k < n) S.hi[which] = probe_at(lo, hi, k, n);
+    if (k > 0) S.lo[which] = probe_at(lo, hi, k - 1, n) + (kFloor ? 1 : 0);
+    S.arrive = 0u;
+  }
+}
+
+// The critical tied group: blocks with th_lo[j] <= imp < th_hi[j].
+__global__ void __launch_bounds__(256) k_alloc_group(const __grid_constant__ AllocArgs a) {
+  AllocState &S = *a.st;
+  const double q = __longlong_as_double(S.lo[0]);
+  const double lam_lo = __longlong_as_double(S.lo[1]), lam_hi = __longlong_as_double(S.hi[1]);
+  __shared__ uint32_t s_hw[kMaxCols / 8];
+  const AllocTensor T = a.t[alloc_tensor(a)];
+  int stride;
+  const uint32_t *hw = stage_high_words(T, s_hw, stride);
+  const int row = (blockIdx.x - T.blk0) * blockDim.x + threadIdx.x;
+  unsigned long long m[kMaxJ - 1];
+#pragma unroll
+  for (int j = 0; j < kMaxJ - 1; ++j) m[j] = 0x7ff0000000000000ull;
+  if (row < T.nrows) {
+    const double rr = T.rho[row];
+    double th[kMaxJ - 1];
+    int c[kMaxJ - 1];
+#pragma unroll
+    for (int j = 0; j < kMaxJ - 1; ++j) th[j] = j < a.J - 1 ? __ddiv_rn(lam_lo, a.slopes[j]) : 0.0;
+    first_blocks<kMaxJ - 1>(T.abar, hw, stride, rr, T.inv[row], q, T.nb, th, a.J - 1, 0u, c);
+#pragma unroll
+    for (int j = 0; j < kMaxJ - 1; ++j)
+      if (j < a.J - 1 && c[j] < T.nb) m[j] = (unsigned long long)__double_as_longlong(imp_at(T.abar, rr, q, c[j]));
+  }
+#pragma unroll
+  for (int j = 0; j < kMaxJ - 1; ++j) {
+    if (j >= a.J - 1) break;
+    for (int o = 16; o > 0; o >>= 1) m[j] = min(m[j], __shfl_xor_sync(0xffffffffu, m[j], o));
+    if ((threadIdx.x & 31) == 0) atomicMin(S.vmin + j, m[j]);
+  }
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x != 0 || atomicAdd(&S.arrive, 1u) != gridDim.x - 1) return;
+  __threadfence();
+  S.arrive = 0u;
+  S.jt = -1;
+  S.ngroups = 0;
+  for (int j = 0; j + 1 < a.J; ++j) {
+    const double vm = __longlong_as_double((long long)__ldcg(S.vmin + j));
+    if (vm < __ddiv_rn(lam_hi, a.slopes[j])) {
+      if (S.ngroups++ == 0) {
+        S.jt = j;
+        S.v = vm;
       }
     }
   }
-  if (a.mode == kVmin) return;
-  if (val && a.per_tensor) atomicAdd(a.per_tensor + ti, val);
-  for (int o = 16; o > 0; o >>= 1) val += __shfl_xor_sync(0xffffffffu, val, o);
-  if ((threadIdx.x & 31) == 0 && val) atomicAdd(a.total, val);
+}
+
+// Per tensor: payload bits at the final thresholds (th_hi with the critical
+// rung's at its group's importance) and the group's blocks.
+__global__ void __launch_bounds__(256) k_alloc_final(const __grid_constant__ AllocArgs a) {
+  const AllocState &S = *a.st;
+  if (S.ngroups != 1) return;
+  const double q = __longlong_as_double(S.lo[0]), lam = __longlong_as_double(S.hi[1]), v = S.v;
+  __shared__ uint32_t s_hw[kMaxCols / 8];
+  const int ti = alloc_tensor(a);
+  const AllocTensor T = a.t[ti];
+  int stride;
+  const uint32_t *hw = stage_high_words(T, s_hw, stride);
+  const int row = (blockIdx.x - T.blk0) * blockDim.x + threadIdx.x;
+  unsigned long long bits = 0, tied = 0;
+  if (row < T.nrows) {
+    const double rr = T.rho[row];
+    // Thresholds 0..J-2, then the group's importance again, strictly.
+    double th[kMaxJ];
+    int c[kMaxJ];
+#pragma unroll
+    for (int j = 0; j < kMaxJ; ++j) th[j] = j < a.J - 1 ? (j == S.jt ? v : __ddiv_rn(lam, a.slopes[j])) : v;
+    first_blocks<kMaxJ>(T.abar, hw, stride, rr, T.inv[row], q, T.nb, th, a.J, 1u << (a.J - 1), c);
+    bits = (unsigned long long)a.L[0] * (unsigned long long)T.nb;
+    int above = 0, at = 0;
+#pragma unroll
+    for (int j = 0; j < kMaxJ; ++j) {
+      if (j < a.J - 1) bits += (unsigned long long)(a.L[j + 1] - a.L[j]) * (unsigned long long)(T.nb - c[j]);
+      if (j == S.jt) at = c[j];
+      if (j == a.J - 1) above = c[j];
+    }
+    const unsigned long long mult = T.nrows == 1 ? (unsigned long long)T.R : 1ull;
+    bits *= mult;
+    tied = (unsigned long long)(above - at) * mult;
+  }
+  for (int o = 16; o > 0; o >>= 1) {
+    bits += __shfl_xor_sync(0xffffffffu, bits, o);
+    tied += __shfl_xor_sync(0xffffffffu, tied, o);
+  }
+  if ((threadIdx.x & 31) == 0 && bits) {
+    atomicAdd(a.bits + ti, bits);
+    if (tied) atomicAdd(a.tied + ti, tied);
+  }
+}
+
+template <bool kFloor>
+cudaError_t launch_round(const AllocArgs &A, dim3 grid, bool after_round, cudaStream_t st) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(256);
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = after_round ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, k_alloc_round<kFloor>, A);
 }
 
 double from_bits(int64_t p) {
@@ -1032,56 +1366,6 @@ double from_bits(int64_t p) {
   memcpy(&d, &p, sizeof d);
   return d;
 }
-
-int64_t to_bits(double d) {
-  int64_t p;
-  memcpy(&p, &d, sizeof p);
-  return p;
-}
-
-struct Allocator {
-  AllocArgs base;
-  cudaStream_t st;
-  unsigned long long *dev;  // 1 + nt + kMaxJ counters
-  int nt;
-  seedq_status err = SEEDQ_OK;
-
-  // One evaluation: returns the total; per-tensor counts into pt when given.
-  uint64_t run(int mode, double q, double v, const double *th, uint64_t *pt = nullptr,
-               double *vmin = nullptr) {
-    if (err != SEEDQ_OK) return 0;
-    AllocArgs a = base;
-    a.mode = mode;
-    a.q = q;
-    a.v = v;
-    for (int j = 0; j < kMaxJ; ++j) a.th[j] = (th && j + 1 < a.J) ? th[j] : 0.0;
-    a.total = dev;
-    a.per_tensor = pt ? dev + 1 : nullptr;
-    a.vmin = dev + 1 + nt;
-    std::vector<unsigned long long> init(1 + nt + kMaxJ, 0ull);
-    for (int j = 0; j < kMaxJ; ++j) init[1 + nt + j] = (unsigned long long)to_bits(INFINITY);
-    cudaError_t e = cudaMemcpyAsync(dev, init.data(), sizeof(unsigned long long) * init.size(),
-                                    cudaMemcpyHostToDevice, st);
-    if (e == cudaSuccess) {
-      const int64_t blocks = (a.rows + 255) / 256;
-      k_alloc_eval<<<(int)blocks, 256, 0, st>>>(a);
-      e = cudaGetLastError();
-    }
-    if (e == cudaSuccess)
-      e = cudaMemcpyAsync(init.data(), dev, sizeof(unsigned long long) * init.size(),
-                          cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    if (e != cudaSuccess) {
-      err = cuda_fail(e);
-      return 0;
-    }
-    if (pt)
-      for (int t = 0; t < nt; ++t) pt[t] = init[1 + t];
-    if (vmin)
-      for (int j = 0; j + 1 < a.J; ++j) vmin[j] = from_bits((int64_t)init[1 + nt + j]);
-    return init[0];
-  }
-};
 
 }  // namespace
 }  // namespace seedq
@@ -1121,21 +1405,8 @@ extern "C" seedq_status seedq_allocate(const seedq_factor_desc *tensors, int32_t
   }
   cudaStream_t st = (cudaStream_t)cuda_stream;
 
-  // Factors of every tensor, exactly as the plan computes them: one device
-  // allocation, one upload of all a and rho, three launches for all tensors.
-  std::vector<void *> owned;
-  auto cleanup = [&]() {
-    for (void *p : owned) cudaFree(p);
-  };
-  auto dalloc = [&](size_t bytes) -> void * {
-    void *p = nullptr;
-    if (cudaMalloc(&p, bytes) != cudaSuccess) {
-      cudaGetLastError();
-      return nullptr;
-    }
-    owned.push_back(p);
-    return p;
-  };
+  // One device allocation: every tensor's factors (exactly as the plan
+  // computes them), the ranking's scratch and the search's state.
   int64_t n_a = 0, n_rho = 0, n_rows = 0, n_nb = 0;
   for (int t = 0; t < count; ++t) {
     n_a += tensors[t].cols;
@@ -1143,24 +1414,36 @@ extern "C" seedq_status seedq_allocate(const seedq_factor_desc *tensors, int32_t
     n_rows += tensors[t].rows;
     n_nb += tensors[t].cols / 8;
   }
-  std::vector<float> h_in((size_t)(n_a + n_rho));
-  float *d_in = (float *)dalloc(sizeof(float) * (size_t)(n_a + n_rho));
-  int32_t *d_perm = (int32_t *)dalloc(sizeof(int32_t) * (size_t)n_a);
-  double *d_abar = (double *)dalloc(sizeof(double) * (size_t)n_nb);
-  double *d_rho = (double *)dalloc(sizeof(double) * (size_t)n_rows);
-  FacJob *d_jobs = (FacJob *)dalloc(sizeof(FacJob) * count);
-  // Stable column rankings of all tensors in one sort and one rank launch.
-  float *d_skey = (float *)dalloc(sizeof(float) * (size_t)n_a);
-  int32_t *d_sidx = (int32_t *)dalloc(sizeof(int32_t) * (size_t)n_a);
-  RankJob<float> *d_rjobs = (RankJob<float> *)dalloc(sizeof(RankJob<float>) * count);
-  std::vector<RankJob<float>> hr(count);
-  if (!d_in || !d_perm || !d_abar || !d_rho || !d_jobs || !d_skey || !d_sidx || !d_rjobs) {
-    cleanup();
-    return SEEDQ_ERR_NOMEM;
+  size_t bytes = 0;
+  auto take = [&](size_t n) {
+    const size_t o = bytes;
+    bytes += (n + 255) / 256 * 256;
+    return o;
+  };
+  const size_t o_in = take(sizeof(float) * (size_t)(n_a + n_rho)), o_perm = take(sizeof(int32_t) * (size_t)n_a);
+  const size_t o_abar = take(sizeof(double) * (size_t)n_nb), o_rho = take(sizeof(double) * (size_t)n_rows);
+  const size_t o_inv = take(sizeof(double) * (size_t)n_rows);
+  const size_t o_skey = take(sizeof(float) * (size_t)n_a), o_sidx = take(sizeof(int32_t) * (size_t)n_a);
+  const size_t o_jobs = take(sizeof(FacJob) * count), o_rjobs = take(sizeof(RankJob<float>) * count);
+  const size_t o_t = take(sizeof(AllocTensor) * count), o_state = take(sizeof(AllocState));
+  const size_t o_cnt = take(sizeof(uint64_t) * 2 * (size_t)count);
+  uint8_t *base = nullptr;
+  cudaError_t e = cudaMallocAsync((void **)&base, bytes, st);
+  if (e != cudaSuccess) {
+    cudaGetLastError();
+    return e == cudaErrorMemoryAllocation ? SEEDQ_ERR_NOMEM : cuda_fail(e);
   }
+  float *d_in = (float *)(base + o_in);
+  int32_t *d_perm = (int32_t *)(base + o_perm);
+  double *d_abar = (double *)(base + o_abar), *d_rho = (double *)(base + o_rho), *d_inv = (double *)(base + o_inv);
+  AllocState *d_state = (AllocState *)(base + o_state);
+  uint64_t *d_cnt = (uint64_t *)(base + o_cnt);
+  std::vector<float> h_in((size_t)(n_a + n_rho));
+  std::vector<RankJob<float>> hr(count);
   std::vector<FacJob> hj(count);
   std::vector<AllocTensor> ht(count);
   int64_t rows_total = 0;
+  int32_t blocks = 0;
   {
     int64_t oa = 0, orh = n_a, orow = 0, onb = 0;
     for (int t = 0; t < count; ++t) {
@@ -1172,136 +1455,115 @@ extern "C" seedq_status seedq_allocate(const seedq_factor_desc *tensors, int32_t
         rho_dev = d_in + orh;
         orh += d.rows;
       }
-      hj[t] = FacJob{d_in + oa, rho_dev, d_perm + oa, d_abar + onb, d_rho + orow, d.rows,
+      hj[t] = FacJob{d_in + oa, rho_dev, d_perm + oa, d_abar + onb, d_rho + orow, d_inv + orow, d.rows,
                      (int32_t)d.cols};
-      hr[t] = RankJob<float>{d_in + oa, d_perm + oa, d_skey + oa, d_sidx + oa, (int32_t)d.cols, 0, 0};
-      ht[t] = AllocTensor{d_abar + onb, d_rho + orow, d.rows, rows_total, d.rho ? (int32_t)d.rows : 1,
+      hr[t] = RankJob<float>{d_in + oa, d_perm + oa, (float *)(base + o_skey) + oa, (int32_t *)(base + o_sidx) + oa,
+                             (int32_t)d.cols, 0, 0};
+      ht[t] = AllocTensor{d_abar + onb, d_rho + orow, d_inv + orow, d.rows, blocks, d.rho ? (int32_t)d.rows : 1,
                           (int32_t)(d.cols / 8)};
       rows_total += ht[t].nrows;
+      blocks += (ht[t].nrows + 255) / 256;
       oa += d.cols;
       orow += d.rows;
       onb += d.cols / 8;
     }
   }
-  {
-    cudaError_t e = cudaMemcpyAsync(d_in, h_in.data(), sizeof(float) * h_in.size(),
-                                    cudaMemcpyHostToDevice, st);
-    if (e == cudaSuccess)
-      e = cudaMemcpyAsync(d_jobs, hj.data(), sizeof(FacJob) * count, cudaMemcpyHostToDevice, st);
-    if (e == cudaSuccess) e = launch_rank<float, false>(hr.data(), count, d_rjobs, st);
-    if (e == cudaSuccess) {
-      k_factors_multi<<<count, 1024, 0, st>>>(d_jobs);
-      e = cudaGetLastError();
-    }
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);  // h_in is pageable and goes out of scope
-    if (e != cudaSuccess) {
-      cleanup();
-      return cuda_fail(e);
-    }
-  }
-  AllocTensor *dt = (AllocTensor *)dalloc(sizeof(AllocTensor) * count);
-  unsigned long long *dev = (unsigned long long *)dalloc(sizeof(unsigned long long) * (1 + count + kMaxJ));
-  if (!dt || !dev) {
-    cleanup();
-    return SEEDQ_ERR_NOMEM;
-  }
-  {
-    const cudaError_t e =
-        cudaMemcpyAsync(dt, ht.data(), sizeof(AllocTensor) * count, cudaMemcpyHostToDevice, st);
-    if (e != cudaSuccess) {
-      cleanup();
-      return cuda_fail(e);
-    }
-  }
-  Allocator A;
-  memset(&A.base, 0, sizeof A.base);
-  A.base.t = dt;
-  A.base.nt = count;
-  A.base.rows = rows_total;
-  A.base.J = J;
-  for (int j = 0; j < J; ++j) A.base.L[j] = L[j];
-  A.st = st;
-  A.dev = dev;
-  A.nt = count;
-  auto thresholds = [&](double lambda, double *th) {
-    for (int j = 0; j + 1 < J; ++j) th[j] = lambda / slopes[j];
-  };
-  auto finish = [&](seedq_status rc) {
-    cleanup();
-    return A.err != SEEDQ_OK ? A.err : rc;
-  };
-
   // Floor: the m-th smallest raw importance, m = ceil(f N) (positive doubles
-  // order as their bit patterns).
+  // order as their bit patterns).  Multiplier: payload bits <= floor(8 rbar N).
   uint64_t m = (uint64_t)ceil(floor_f * (double)nblocks);
   if (m < 1) m = 1;
-  int64_t lo = 0, hi = to_bits(INFINITY);
-  while (lo < hi && A.err == SEEDQ_OK) {
-    const int64_t mid = lo + (hi - lo) / 2;
-    if (A.run(kCountLE, 0.0, from_bits(mid), nullptr) >= m) hi = mid;
-    else lo = mid + 1;
-  }
-  const double q = from_bits(lo);
-  *q_out = q;
-
-  // Multiplier: bisection on lambda for payload bits <= floor(8 rbar N).
   const uint64_t budget = (uint64_t)floor(8.0 * rbar * (double)nblocks);
-  double th_lo[kMaxJ] = {0}, th_hi[kMaxJ] = {0};
-  std::vector<uint64_t> pt(count);
-  thresholds(INFINITY, th_hi);
-  if (A.run(kBits, q, 0.0, th_hi) > budget) return finish(SEEDQ_ERR_SCHEDULE);
-  thresholds(0.0, th_lo);
-  if (A.run(kBits, q, 0.0, th_lo, pt.data()) <= budget) {  // every block on the top rung
-    for (int j = 0; j + 1 < J; ++j) theta[j] = th_lo[j];
+  // The ends of the multiplier's range need no search: every block on the
+  // lowest rung at infinity, on the top rung at zero.
+  const bool infeasible = (uint64_t)L[0] * nblocks > budget;
+  const bool all_top = !infeasible && (uint64_t)L[J - 1] * nblocks <= budget;
+  AllocState h;
+  memset(&h, 0, sizeof h);
+  const double inf = INFINITY;
+  int64_t inf_bits;
+  memcpy(&inf_bits, &inf, sizeof inf_bits);
+  h.hi[0] = h.hi[1] = inf_bits;
+  for (int j = 0; j < kMaxJ; ++j) h.vmin[j] = (unsigned long long)inf_bits;
+  AllocArgs A;
+  memset(&A, 0, sizeof A);
+  A.t = (const AllocTensor *)(base + o_t);
+  A.nt = count;
+  A.J = J;
+  for (int j = 0; j < J; ++j) A.L[j] = L[j];
+  for (int j = 0; j + 1 < J; ++j) A.slopes[j] = slopes[j];
+  A.st = d_state;
+  A.bits = (unsigned long long *)d_cnt;
+  A.tied = (unsigned long long *)(d_cnt + count);
+  // Probes per round (one less than a power of two): about 2^16 row searches a
+  // round.  A call over 8197 rows (probes 3 / 7 / 15 / 31): 834 / 681 / 702 /
+  // 917 us, 5007 with a host read after each of 133 single steps; 1.3 M rows
+  // (one probe): 26 ms, of which half is the host's checks, against 67.
+  int probes = kMaxProbes;
+  while (probes > 1 && rows_total * probes > (1 << 16)) probes /= 2;
+  int per_round = 0;
+  while ((2 << per_round) <= probes + 1) ++per_round;  // halvings a round makes
+  const int rounds = (63 + per_round - 1) / per_round + 1;
+  const unsigned gx = (unsigned)blocks;
+  std::vector<uint64_t> cnt(2 * (size_t)count, 0);
+  auto up = [&](void *dst, const void *src, size_t n) {
+    if (e == cudaSuccess) e = cudaMemcpyAsync(dst, src, n, cudaMemcpyHostToDevice, st);
+  };
+  up(d_in, h_in.data(), sizeof(float) * h_in.size());
+  up(base + o_jobs, hj.data(), sizeof(FacJob) * count);
+  up(base + o_t, ht.data(), sizeof(AllocTensor) * count);
+  up(d_state, &h, sizeof h);
+  if (e == cudaSuccess) e = cudaMemsetAsync(d_cnt, 0, sizeof(uint64_t) * 2 * (size_t)count, st);
+  if (e == cudaSuccess) e = launch_rank<float, false>(hr.data(), count, (RankJob<float> *)(base + o_rjobs), st);
+  if (e == cudaSuccess) {
+    k_factors_multi<<<2 * count, 1024, 0, st>>>((const FacJob *)(base + o_jobs));
+    A.target = m;
+    for (int r = 0; r < rounds && e == cudaSuccess; ++r) e = launch_round<true>(A, dim3(gx, probes), r > 0, st);
+    if (!infeasible && !all_top) {
+      A.target = budget;
+      for (int r = 0; r < rounds && e == cudaSuccess; ++r) e = launch_round<false>(A, dim3(gx, probes), true, st);
+      k_alloc_group<<<gx, 256, 0, st>>>(A);
+      k_alloc_final<<<gx, 256, 0, st>>>(A);
+    }
+    if (e == cudaSuccess) e = cudaGetLastError();
+  }
+  if (e == cudaSuccess) e = cudaMemcpyAsync(&h, d_state, sizeof h, cudaMemcpyDeviceToHost, st);
+  if (e == cudaSuccess)
+    e = cudaMemcpyAsync(cnt.data(), d_cnt, sizeof(uint64_t) * cnt.size(), cudaMemcpyDeviceToHost, st);
+  // The host's arrays go out of scope: the copies from them have to be done.
+  const cudaError_t es = cudaStreamSynchronize(st);
+  if (e == cudaSuccess) e = es;
+  const cudaError_t ef = cudaFreeAsync(base, st);
+  if (e == cudaSuccess) e = ef;
+  if (e != cudaSuccess) return cuda_fail(e);
+  *q_out = from_bits(h.lo[0]);
+  if (infeasible) return SEEDQ_ERR_SCHEDULE;
+  if (all_top) {
+    for (int j = 0; j + 1 < J; ++j) theta[j] = 0.0 / slopes[j];
     *j_tie = -1;
     for (int t = 0; t < count; ++t) {
       tie_count[t] = 0;
-      stream_bits[t] = pt[t];
+      stream_bits[t] = (uint64_t)L[J - 1] * (uint64_t)tensors[t].rows * (uint64_t)(tensors[t].cols / 8);
     }
-    return finish(SEEDQ_OK);
+    return SEEDQ_OK;
   }
-  lo = 0;
-  hi = to_bits(INFINITY);
-  while (hi - lo > 1 && A.err == SEEDQ_OK) {  // bits(lo) > budget >= bits(hi)
-    const int64_t mid = lo + (hi - lo) / 2;
-    double th[kMaxJ];
-    thresholds(from_bits(mid), th);
-    if (A.run(kBits, q, 0.0, th) > budget) lo = mid;
-    else hi = mid;
-  }
-  thresholds(from_bits(lo), th_lo);
-  thresholds(from_bits(hi), th_hi);
-
-  // The critical tied group: blocks with th_lo[j] <= imp < th_hi[j].
-  double vmin[kMaxJ];
-  A.run(kVmin, q, 0.0, th_lo, nullptr, vmin);
-  int jt = -1;
-  double v = 0.0;
-  for (int j = 0; j + 1 < J; ++j) {
-    if (vmin[j] < th_hi[j]) {
-      if (jt >= 0) return finish(SEEDQ_ERR_SCHEDULE);
-      jt = j;
-      v = vmin[j];
-    }
-  }
-  if (jt < 0) return finish(SEEDQ_ERR_SCHEDULE);
-  for (int j = 0; j + 1 < J; ++j) theta[j] = th_hi[j];
-  theta[jt] = v;
-  const uint64_t b_hi = A.run(kBits, q, 0.0, theta, pt.data());
-  const uint64_t step = (uint64_t)(L[jt + 1] - L[jt]);
-  const uint64_t excess = b_hi > budget ? b_hi - budget : 0;
-  uint64_t T = (excess + step - 1) / step;
+  if (h.ngroups != 1) return SEEDQ_ERR_SCHEDULE;
+  const double lam_hi = from_bits(h.hi[1]);
+  for (int j = 0; j + 1 < J; ++j) theta[j] = lam_hi / slopes[j];
+  theta[h.jt] = h.v;
   // App. A.5: demote members of the group in block order (tensor order, then
   // row-major within a tensor) until the budget is met.
-  std::vector<uint64_t> tied(count, 0);
-  if (T) A.run(kTied, q, v, nullptr, tied.data());
+  uint64_t b_hi = 0;
+  for (int t = 0; t < count; ++t) b_hi += cnt[t];
+  const uint64_t step = (uint64_t)(L[h.jt + 1] - L[h.jt]);
+  const uint64_t excess = b_hi > budget ? b_hi - budget : 0;
+  uint64_t T = (excess + step - 1) / step;
   for (int t = 0; t < count; ++t) {
-    const uint64_t d = T < tied[t] ? T : tied[t];
+    const uint64_t tied = cnt[(size_t)count + t], d = T < tied ? T : tied;
     tie_count[t] = (int64_t)d;
     T -= d;
-    stream_bits[t] = pt[t] - d * step;
+    stream_bits[t] = cnt[t] - d * step;
   }
-  if (T != 0) return finish(SEEDQ_ERR_SCHEDULE);
-  *j_tie = jt;
-  return finish(SEEDQ_OK);
+  if (T != 0) return SEEDQ_ERR_SCHEDULE;
+  *j_tie = h.jt;
+  return SEEDQ_OK;
 }
