@@ -1,6 +1,6 @@
 // Fused reconstruction x matrix-vector product: y = W_hat x, and the decode-batch
-// skinny GEMM Y = X W_hat^T (n <= 16), for one tensor or for several tensors
-// in one launch (the tensors of a decode step are independent: Alg. 2 decodes
+// skinny GEMM Y = X W_hat^T (n <= 16; batches above four on the tensor cores,
+// gemm_mma.cuh), for one tensor or for several tensors in one launch (the tensors of a decode step are independent: Alg. 2 decodes
 // each tensor on its own, in no fixed order).  W_hat is never written to memory; HBM carries only
 // the compressed streams, the plan rows and x / y.
 //
@@ -23,6 +23,7 @@
 #include <cuda_fp16.h>
 #include <string.h>
 
+#include <algorithm>
 #include <cstddef>
 #include <new>
 #include <vector>
@@ -44,8 +45,9 @@ struct Cfg {
   // Columns per stage and row groups per round: the widest stage for which
   // 12 warps' double buffers, the jump tables and the round's partial sums
   // fit in shared memory (wider stages amortize staging and bookkeeping).
-  static constexpr int ST = NB == 1 ? 27 : NB == 2 ? 21 : NB == 4 ? 15 : NB == 8 ? 12 : 7;
-  static constexpr int RG = NB == 1 ? 8 : NB <= 4 ? 4 : 1;
+  static_assert(NB <= 4, "larger batches run on the tensor cores");
+  static constexpr int ST = NB == 1 ? 27 : NB == 2 ? 21 : 15;
+  static constexpr int RG = NB == 1 ? 8 : 4;
   // 16-byte pieces per staged row: ST blocks of at most 44 bits, the 96-bit
   // read-ahead of the last block, and up to 15 + 15 bytes of alignment.
   static constexpr int PIECES = (ST * 44 / 8 + 12 + 30 + 15) / 16 + 1;
@@ -61,7 +63,8 @@ struct TensorArgs {
   LayerArgs p;
   const uint16_t *x;      // n x C bf16, original column order
   float *y;               // n x R
-  int64_t ubegin;         // first unit of this tensor in the launch's sequence
+  int64_t ubegin;         // first unit of this tensor in the launch's sequence (32-row groups)
+  int64_t ubegin_mm;      // the same for the tensor-core kernel (superblocks)
   uint64_t stream_bytes;  // readable bytes of the bound stream buffer
   int64_t cpre, rpre;     // layer sets: columns and rows of the tensors before it
 };
@@ -82,6 +85,13 @@ struct MultiArgs {
   const uint16_t *Xall;    // layer set: x of tensor i at Xall + n * cpre_i
   float *Yall;             // layer set: y of tensor i at Yall + n * rpre_i
 };
+
+// Batch templates of up to four run on the FMA pipes (k_gemv), larger ones on
+// the tensor cores (k_gemm).  Measured, k_gemv / k_gemm: a 7B layer at 4.0 bits
+// b4 182 / 232 us, b8 261 / 233, b16 381 / 268; at 3.0 bits b4 166 / 205, b8 265
+// / 217, b16 397 / 250; 1024 x 1024 b8 28 / 19, b16 48 / 39; 256 x 256 b8 35 /
+// 19; 1997 x 2072 b8 31 / 29, b16 48 / 38; 11008 x 128 b16 47 / 31.
+__host__ __device__ constexpr bool on_tensor_cores(int NB) { return NB >= 8; }
 
 __host__ __device__ inline int batch_template(int n) {
   return n <= 1 ? 1 : n <= 2 ? 2 : n <= 4 ? 4 : n <= 8 ? 8 : 16;
@@ -592,6 +602,12 @@ __global__ void __launch_bounds__(kThreads, 1) k_gemv(const __grid_constant__ Mu
   }
 }
 
+}  // namespace seedq
+
+#include "gemm_mma.cuh"
+
+namespace seedq {
+
 // Activations in permuted column order, zero at outlier columns (their
 // contribution is added exactly by the epilogue), weight-major with NB values
 // per weight: xperm[p * NB + b] = x_b[perm[p]] (0 for b >= n).  One grid row
@@ -652,10 +668,36 @@ __global__ void k_xperm_set(const TensorArgs *__restrict__ tens, const uint16_t 
   }
 }
 
+// The same for the tensor cores' layout.
+__global__ void k_xperm_mm(const __grid_constant__ XpermArgs a) {
+  asm volatile("griddepcontrol.launch_dependents;");
+  const auto &T = a.t[blockIdx.y];
+  xperm_bf16(T.perm, T.x, reinterpret_cast<uint4 *>(T.xperm), T.C, T.n_out, T.out_cols, a.n, a.nbt);
+}
+
+__global__ void k_xperm_mm_set(const TensorArgs *__restrict__ tens, const uint16_t *Xall, int n, int nbt) {
+  asm volatile("griddepcontrol.launch_dependents;");
+  const TensorArgs &T = tens[blockIdx.y];
+  const LayerArgs &p = T.p;
+  xperm_bf16(p.perm, Xall + (int64_t)n * T.cpre, reinterpret_cast<uint4 *>(p.xperm), p.C, p.n_out, p.out_cols, n, nbt);
+}
+
 template <int NB>
 static size_t smem_bytes() {
-  return sizeof(uint64_t) * 512 * kTableSlots + (size_t)kWarps * Cfg<NB>::WARP_BYTES +
-         sizeof(float) * Cfg<NB>::RG * kWarps * 32 * NB + sizeof(uint4) * Cfg<NB>::RG * 32 * 2;
+  if constexpr (on_tensor_cores(NB)) {
+    return MmCfg<NB>::SMEM;
+  } else {
+    return sizeof(uint64_t) * 512 * kTableSlots + (size_t)kWarps * Cfg<NB>::WARP_BYTES +
+           sizeof(float) * Cfg<NB>::RG * kWarps * 32 * NB + sizeof(uint4) * Cfg<NB>::RG * 32 * 2;
+  }
+}
+
+using FusedKernel = void (*)(MultiArgs);
+
+template <int NB, bool kSet>
+static FusedKernel fused_kernel() {
+  if constexpr (on_tensor_cores(NB)) return k_gemm<NB, kSet>;
+  else return k_gemv<NB, kSet>;
 }
 
 // The fused kernel's dynamic shared-memory limit is a per-device attribute:
@@ -670,7 +712,7 @@ static DeviceOnce &smem_once() {
 template <int NB, bool kSet>
 static cudaError_t set_smem_limit(int dev) {
   return (cudaError_t)smem_once<NB, kSet>().run(dev, [] {
-    return (int)cudaFuncSetAttribute(k_gemv<NB, kSet>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    return (int)cudaFuncSetAttribute(fused_kernel<NB, kSet>(), cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      (int)smem_bytes<NB>());
   });
 }
@@ -680,12 +722,12 @@ static cudaError_t launch_fused(const cudaLaunchConfig_t &cfg, const MultiArgs &
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = set_smem_limit<NB, kSet>(dev);
-  if (e == cudaSuccess) e = cudaLaunchKernelEx(&cfg, k_gemv<NB, kSet>, a);
+  if (e == cudaSuccess) e = cudaLaunchKernelEx(&cfg, fused_kernel<NB, kSet>(), a);
   if (e == cudaErrorInvalidValue) {
     (void)cudaGetLastError();
     smem_once<NB, kSet>().forget(dev);
     e = set_smem_limit<NB, kSet>(dev);
-    if (e == cudaSuccess) e = cudaLaunchKernelEx(&cfg, k_gemv<NB, kSet>, a);
+    if (e == cudaSuccess) e = cudaLaunchKernelEx(&cfg, fused_kernel<NB, kSet>(), a);
   }
   return e;
 }
@@ -697,13 +739,19 @@ static cudaError_t launch_fused(const cudaLaunchConfig_t &cfg, const MultiArgs &
 // places all cuts in order.
 static void partition(const seedq_layer *const *layers, int nt, int n, int64_t *ubegin, int64_t *cta_begin,
                       int &ctas_out) {
+  // A unit's rows: one group of 32, or a superblock of them on the tensor cores.
+  const int gs = on_tensor_cores(batch_template(n)) ? kMmGroups : 1;
   const double cb = cost_block(n);
-  auto gcost = [&](const seedq_layer *L, int64_t g) { return kCostK * L->h_gk[g] + cb * L->h_gp[g]; };
+  auto groups = [&](const seedq_layer *L) { return ((L->args.R + 31) / 32 + gs - 1) / gs; };
+  auto gcost = [&](const seedq_layer *L, int64_t g) {
+    const int64_t i = std::min(g * gs, (L->args.R + 31) / 32);
+    return gs > 1 ? kCostK * L->h_mk[i] + cb * L->h_mp[i] : kCostK * L->h_gk[i] + cb * L->h_gp[i];
+  };
   int64_t U = 0;
   double total = 0.0;
   for (int i = 0; i < nt; ++i) {
     const seedq_layer *L = layers[i];
-    const int64_t G = (L->args.R + 31) / 32;
+    const int64_t G = groups(L);
     ubegin[i] = U;
     U += G * L->args.nb;
     total += gcost(L, G);
@@ -718,13 +766,13 @@ static void partition(const seedq_layer *const *layers, int nt, int n, int64_t *
   double tbase = 0.0;  // cost of the tensors before the current one
   for (int ti = 0; ti < nt && c < ctas; ++ti) {
     const seedq_layer *L = layers[ti];
-    const int64_t G = (L->args.R + 31) / 32;
+    const int64_t G = groups(L);
     const int J = L->args.J, Jm1 = J > 1 ? J - 1 : 1, nb = L->args.nb;
     for (int64_t g = 0; g < G && c < ctas; ++g) {
       const double g0 = gcost(L, g), g1 = gcost(L, g + 1);
       double target = total * c / ctas;
       if (target - tbase >= g1) continue;
-      const int32_t *b = L->h_repbk + g * Jm1;
+      const int32_t *b = L->h_repbk + g * gs * Jm1;
       double rep = 0.0;
       for (int j = 0, clo = 0; j < J; ++j) {
         const int chi = (j < J - 1) ? b[j] : nb;
@@ -736,16 +784,26 @@ static void partition(const seedq_layer *const *layers, int nt, int n, int64_t *
         const double lt = target - tbase;
         double acc = g0;
         int col = nb, clo = 0;
-        for (int j = 0; j < J; ++j) {
-          const int chi = (j < J - 1) ? b[j] : nb;
-          const double per = (kCostK * L->k[j] + cb) * scale;
-          const double seg = per * (chi - clo);
-          if (acc + seg > lt) {
-            col = clo + (int)((lt - acc) / per);
-            break;
+        if (gs > 1) {  // by the superblock's work profile
+          const float *prof = L->h_prof + g * 2 * (kProfile + 1);
+          auto at = [&](int i) { return g0 + kCostK * prof[kProfile + 1 + i] + cb * prof[i]; };
+          int i = 1;
+          while (i < kProfile && at(i) <= lt) ++i;
+          const double c0 = at(i - 1), c1 = at(i);
+          const int b0 = (int)((int64_t)nb * (i - 1) / kProfile), b1 = (int)((int64_t)nb * i / kProfile);
+          col = b0 + (c1 > c0 ? (int)((lt - c0) / (c1 - c0) * (b1 - b0)) : 0);
+        } else {
+          for (int j = 0; j < J; ++j) {
+            const int chi = (j < J - 1) ? b[j] : nb;
+            const double per = (kCostK * L->k[j] + cb) * scale;
+            const double seg = per * (chi - clo);
+            if (acc + seg > lt) {
+              col = clo + (int)((lt - acc) / per);
+              break;
+            }
+            acc += seg;
+            clo = chi;
           }
-          acc += seg;
-          clo = chi;
         }
         if (col < 0) col = 0;
         if (col > nb) col = nb;
@@ -783,7 +841,7 @@ static seedq_status launch(const seedq_layer *const *layers, int nt, const uint1
   }
   int64_t ub[kMaxTensors];
   partition(layers, nt, n, ub, a->cta_begin, a->ctas);
-  for (int i = 0; i < nt; ++i) a->t[i].ubegin = ub[i];
+  for (int i = 0; i < nt; ++i) a->t[i].ubegin = a->t[i].ubegin_mm = ub[i];
   a->tens = nullptr;
   a->cbd = nullptr;
   a->Xall = nullptr;
@@ -806,7 +864,8 @@ static seedq_status launch(const seedq_layer *const *layers, int nt, const uint1
     }
     const int64_t want = ((int64_t)NB * maxC + 255) / 256;
     const int gx = (int)(want < 64 ? want : 64);
-    k_xperm<<<dim3(gx, nt), 256, 0, st>>>(xa);
+    if constexpr (on_tensor_cores(NB)) k_xperm_mm<<<dim3(gx, nt), 256, 0, st>>>(xa);
+    else k_xperm<<<dim3(gx, nt), 256, 0, st>>>(xa);
     cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess) {
       // Programmatic dependent launch: the fused kernel's CTAs may start (and
@@ -814,7 +873,7 @@ static seedq_status launch(const seedq_layer *const *layers, int nt, const uint1
       // its writes before the first activation load.
       cudaLaunchConfig_t cfg = {};
       cfg.gridDim = dim3(a->ctas);
-      cfg.blockDim = dim3(kThreads);
+      cfg.blockDim = dim3(on_tensor_cores(NB) ? kMmThreads : kThreads);
       cfg.dynamicSmemBytes = smem_bytes<NB>();
       cfg.stream = st;
       cudaLaunchAttribute attr[1];
@@ -881,12 +940,13 @@ static seedq_status launch_set(const seedq_layer_set *S, const uint16_t *X, int 
   a.Yall = Y;
   const int64_t want = ((int64_t)NB * S->maxC + 255) / 256;
   const int gx = (int)(want < 64 ? want : 64);
-  k_xperm_set<<<dim3(gx, S->nt), 256, 0, st>>>(S->d_tens, X, n, NB);
+  if constexpr (on_tensor_cores(NB)) k_xperm_mm_set<<<dim3(gx, S->nt), 256, 0, st>>>(S->d_tens, X, n, NB);
+  else k_xperm_set<<<dim3(gx, S->nt), 256, 0, st>>>(S->d_tens, X, n, NB);
   cudaError_t e = cudaGetLastError();
   if (e == cudaSuccess) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(a.ctas);
-    cfg.blockDim = dim3(kThreads);
+    cfg.blockDim = dim3(on_tensor_cores(NB) ? kMmThreads : kThreads);
     cfg.dynamicSmemBytes = smem_bytes<NB>();
     cfg.stream = st;
     cudaLaunchAttribute attr[1];
@@ -936,7 +996,7 @@ seedq_status seedq_layer_set_create(const seedq_layer *const *layers, int32_t co
   S->cols = S->cpre[count];
   S->rows = S->rpre[count];
   std::vector<TensorArgs> h(count);
-  std::vector<int64_t> ub(count), cta(kMaxCtas + 1);
+  std::vector<int64_t> ub(count), ub1(count), ub_mm(count), cta(kMaxCtas + 1);
   seedq_status rc = SEEDQ_OK;
   cudaError_t e = cudaSuccess;
   for (int k = 0; k < 5 && rc == SEEDQ_OK && e == cudaSuccess; ++k) {
@@ -945,6 +1005,7 @@ seedq_status seedq_layer_set_create(const seedq_layer *const *layers, int32_t co
     int ctas = 0;
     partition(layers, count, nb, ub.data(), cta.data(), ctas);
     S->ctas[k] = ctas;
+    (on_tensor_cores(nb) ? ub_mm : ub1) = ub;
     e = cudaMalloc((void **)&S->d_cta[k], sizeof(int64_t) * (ctas + 1));
     if (e == cudaSuccess)
       e = cudaMemcpy(S->d_cta[k], cta.data(), sizeof(int64_t) * (ctas + 1), cudaMemcpyHostToDevice);
@@ -952,7 +1013,8 @@ seedq_status seedq_layer_set_create(const seedq_layer *const *layers, int32_t co
   for (int i = 0; i < count; ++i) {
     memset(&h[i], 0, sizeof(TensorArgs));
     h[i].p = layers[i]->args;
-    h[i].ubegin = ub[i];
+    h[i].ubegin = ub1[i];
+    h[i].ubegin_mm = ub_mm[i];
     h[i].stream_bytes = layers[i]->stream_bytes;
     h[i].cpre = S->cpre[i];
     h[i].rpre = S->rpre[i];

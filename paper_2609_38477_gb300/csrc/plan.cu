@@ -522,6 +522,9 @@ static void free_layer(seedq_layer *L) {
   cudaFree(L->d_xperm);
   free(L->h_gp);
   free(L->h_gk);
+  free(L->h_mp);
+  free(L->h_mk);
+  free(L->h_prof);
   free(L->h_repbk);
 
   free(L);
@@ -545,11 +548,15 @@ static seedq_status build_costs(seedq_layer *L, cudaStream_t st) {
   int32_t *brk = (int32_t *)malloc(sizeof(int32_t) * R * Jm1);
   L->h_gp = (double *)malloc(sizeof(double) * (G + 1));
   L->h_gk = (double *)malloc(sizeof(double) * (G + 1));
+  L->h_mp = (double *)malloc(sizeof(double) * (G + 1));
+  L->h_mk = (double *)malloc(sizeof(double) * (G + 1));
+  const int64_t SB = (G + kMmGroups - 1) / kMmGroups;
+  L->h_prof = (float *)calloc((size_t)SB * 2 * (kProfile + 1), sizeof(float));
   L->h_repbk = (int32_t *)malloc(sizeof(int32_t) * G * Jm1);
   const int nst = (nb + kCostStage - 1) / kCostStage;
   uint8_t *mixed = (uint8_t *)malloc(nst);
   seedq_status rc = SEEDQ_OK;
-  if (!rowperm || !brk || !L->h_gp || !L->h_gk || !L->h_repbk || !mixed) rc = SEEDQ_ERR_NOMEM;
+  if (!rowperm || !brk || !L->h_gp || !L->h_gk || !L->h_mp || !L->h_mk || !L->h_prof || !L->h_repbk || !mixed) rc = SEEDQ_ERR_NOMEM;
   cudaError_t e = cudaSuccess;
   if (rc == SEEDQ_OK) e = cudaMemcpyAsync(rowperm, L->d_rowperm, sizeof(int32_t) * R, cudaMemcpyDeviceToHost, st);
   if (rc == SEEDQ_OK && e == cudaSuccess && J > 1)
@@ -559,7 +566,11 @@ static seedq_status build_costs(seedq_layer *L, cudaStream_t st) {
   if (rc == SEEDQ_OK) {
     L->h_gp[0] = 0.0;
     L->h_gk[0] = 0.0;
+    L->h_mp[0] = 0.0;
+    L->h_mk[0] = 0.0;
     const int32_t *rowb[32];
+    int32_t last_bk[kMaxJ] = {0};
+    bool last_uniform = false;
     for (int64_t g = 0; g < G; ++g) {
       int nr = 0;
       for (int i = 0; i < 32 && g * 32 + i < R; ++i) rowb[nr++] = brk + (int64_t)rowperm[g * 32 + i] * Jm1;
@@ -574,6 +585,61 @@ static seedq_status build_costs(seedq_layer *L, cudaStream_t st) {
         K += (double)L->k[j] * (hi - lo);
         lo = hi;
       }
+      // The tensor-core kernel passes, for each set of sixteen rows, over
+      // every column one of them has at a rung; a pass of the group's 32 rows
+      // over a stage costs about five columns more (fitted to per-CTA times).
+      double mP = 0.0, mK = 0.0;
+      float *prof = L->h_prof + (g / kMmGroups) * 2 * (kProfile + 1);
+      constexpr double kPass = 5.0;
+      auto add = [&](int from, int to, double wp, double wk) {
+        mP += wp * (to - from);
+        mK += wk * (to - from);
+        for (int i = 1; i <= kProfile; ++i) {
+          const int c = (int)((int64_t)nb * i / kProfile), n = (c < to ? c : to) - from;
+          if (n <= 0) continue;
+          prof[i] += (float)(wp * n);
+          prof[kProfile + 1 + i] += (float)(wk * n);
+        }
+      };
+      // A group whose rows all have the last one's breakpoints repeats its
+      // profile (tensors without a row factor: every group).
+      bool same = g > 0 && g % kMmGroups != 0;
+      for (int i = 0; i < nr && same; ++i)
+        for (int j = 0; j < J - 1; ++j) same = same && rowb[i][j] == last_bk[j];
+      if (L->max_batch <= 4) {
+        // (never launched)
+      } else if (same && last_uniform) {
+        mP = L->h_mp[g] - L->h_mp[g - 1];
+        mK = L->h_mk[g] - L->h_mk[g - 1];
+        const float f = (float)(g % kMmGroups + 1) / (float)(g % kMmGroups);
+        for (int i = 0; i < 2 * (kProfile + 1); ++i) prof[i] *= f;
+      } else {
+        for (int j = 0; j < J; ++j) {
+          int from32 = nb, to32 = 0;
+          for (int s0 = 0; s0 < nr; s0 += 16) {
+            int from = nb, to = 0;
+            for (int i = s0; i < nr && i < s0 + 16; ++i) {
+              const int a = (j > 0) ? rowb[i][j - 1] : 0, z = (j < J - 1) ? rowb[i][j] : nb;
+              if (a < z) {
+                from = a < from ? a : from;
+                to = z > to ? z : to;
+              }
+            }
+            if (from < to) add(from, to, 0.5, 0.5 * L->k[j]);
+            from32 = from < from32 ? from : from32;
+            to32 = to > to32 ? to : to32;
+          }
+          // One pass per stage it touches: len / 24 of them, and one more.
+          if (from32 < to32) add(from32, to32, kPass / kCostStage + kPass / (to32 - from32), 0.0);
+        }
+        last_uniform = nr == 32;
+        for (int j = 0; j < J - 1; ++j) {
+          last_bk[j] = rowb[0][j];
+          for (int i = 1; i < nr; ++i) last_uniform = last_uniform && rowb[i][j] == rowb[0][j];
+        }
+      }
+      L->h_mp[g + 1] = L->h_mp[g] + mP;
+      L->h_mk[g + 1] = L->h_mk[g] + mK;
       // Stages where the rows' breakpoints differ: replace the first row's
       // passes there by the per-rung maxima over the rows.
       bool any = false;
@@ -762,9 +828,9 @@ seedq_status seedq_layer_prepare(const seedq_layer_desc *d, const seedq_schedule
   ALLOC(L->d_rowperm, sizeof(int32_t) * R);
   ALLOC(L->d_rowrec, sizeof(uint4) * 2 * R);
   ALLOC(L->d_counters, sizeof(int32_t) * ngroups);
-  ALLOC(L->d_slots, sizeof(float) * L->max_ctas * 2 * 32 * kMaxBatch);
   // Weight-major activations, padded to the kernel's batch template.
   const int mbt = mb <= 1 ? 1 : mb <= 2 ? 2 : mb <= 4 ? 4 : mb <= 8 ? 8 : 16;
+  ALLOC(L->d_slots, sizeof(float) * L->max_ctas * 2 * (size_t)slot_floats(mbt));
   ALLOC(L->d_xperm, sizeof(float) * C * mbt);
 
 #undef ALLOC

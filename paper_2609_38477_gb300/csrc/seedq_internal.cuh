@@ -43,7 +43,7 @@ struct LayerArgs {
                             // count (word 6)
   float *xperm;             // C x n: activations in permuted order, weight-major
   int32_t *counters;        // row groups: arrivals of partial sums (0 between calls)
-  float *slots;             // max_ctas x 2 x 32 x 16 partial sums of row groups
+  float *slots;             // max_ctas x 2 partial sums of cut row groups or superblocks
   uint32_t *flags;
   int64_t R, C;
   int32_t nb;               // C / 8 blocks per row
@@ -67,10 +67,16 @@ namespace seedq {
 // single-rung tensors (S = 8..16, k = 2..6; n = 1, 4, 16; 2 and 8 between).
 constexpr double kCostK = 1.0;
 inline double cost_block(int n) {
-  return n <= 1 ? 3.7 : n <= 2 ? 5.3 : n <= 4 ? 8.4 : n <= 8 ? 12.5 : 19.6;
+  return n <= 1 ? 3.7 : n <= 2 ? 5.3 : n <= 4 ? 8.4 : 8.0;
 }
 // Stage width (blocks) the work profile assumes.
 constexpr int kCostStage = 24;
+// Columns at which a superblock's work profile is kept.
+constexpr int kProfile = 16;
+constexpr int kMmGroups = 4;  // row groups of a superblock
+// Floats of one CTA's partial sums of a cut group (k_gemv: 32 rows) or
+// superblock (k_gemm: 128 rows) at batch template nb.
+inline int slot_floats(int nb) { return nb > 4 ? 128 * nb : 32 * kMaxBatch; }
 }  // namespace seedq
 
 struct seedq_layer {
@@ -100,6 +106,10 @@ struct seedq_layer {
   // Host-side work profile of the fused kernel, per row group (G + 1 entries,
   // cumulative): block passes the warp makes, and the sum of k over them.
   double *h_gp, *h_gk;
+  double *h_mp, *h_mk;   // the same for the tensor-core kernel
+  // Per superblock, the share of those before column nb * i / kProfile (passes,
+  // then the sum of k): kProfile + 1 entries each.
+  float *h_prof;
   int32_t *h_repbk;      // host: breakpoints of each row group's first row (G x (J-1))
   uint64_t *d_row_off;
   uint64_t *d_tables;
