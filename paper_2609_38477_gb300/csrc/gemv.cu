@@ -38,6 +38,7 @@ namespace seedq {
 constexpr int kWarps = 12;
 constexpr int kThreads = kWarps * 32;
 constexpr int kMaxTensors = 8;
+constexpr int kMinStage = 2;  // columns per stage of a short round, at least
 constexpr int kMaxCtas = 256;
 
 template <int NB>
@@ -230,16 +231,17 @@ struct Piece {
 // round-robin to the CTA's warps; lane = row of the stage's row group.  Each
 // buffer slot carries the row data of the stage staged into it.  A warp's sums
 // go to comb[piece][warp][lane] whenever its next stage is in another piece.
-template <int NB>
+template <int NB, bool kShort>
 __device__ __forceinline__ void warp_round(const TensorArgs &T, int n, const uint4 *rdn,
                                            const uint64_t *tabs, uint32_t *sbuf, float *xbuf,
                                            const uint4 *rrec, const Piece *pcs, const int *pst, int np,
-                                           int nst_total,
+                                           int nst_total, int st_short,
                                            float *comb, int warp, int lane) {
   using CF = Cfg<NB>;
   const LayerArgs &p = T.p;
   const int J = p.J, nb = p.nb;
   if (warp >= nst_total) return;
+  const int st = kShort ? st_short : CF::ST;
   const uint8_t *gstream = reinterpret_cast<const uint8_t *>(p.stream);
   int piece_of[2] = {0, 0}, cs_of[2] = {0, 0}, ce_of[2] = {0, 0};
   int jr_of[2] = {0, 0}, nxt_of[2] = {0, 0};
@@ -249,7 +251,7 @@ __device__ __forceinline__ void warp_round(const TensorArgs &T, int n, const uin
   auto issue = [&](int t, int sb) {
     while (pi_cur + 1 < np && t >= pst[pi_cur + 1]) ++pi_cur;
     const int pi = pi_cur;
-    const int cs = pcs[pi].ca + (t - pst[pi]) * CF::ST, ce = min(pcs[pi].cb, cs + CF::ST);
+    const int cs = pcs[pi].ca + (t - pst[pi]) * st, ce = min(pcs[pi].cb, cs + st);
     // The lane's row record (bit offset, breakpoints), staged for the round.
     const uint4 m0 = rrec[(pi * 32 + lane) * 2], m1 = rrec[(pi * 32 + lane) * 2 + 1];
     const uint64_t roff = (uint64_t)m0.x | ((uint64_t)m0.y << 32);
@@ -394,7 +396,9 @@ __device__ __forceinline__ float outlier_term(const LayerArgs &p, const uint16_t
 // shared memory; otherwise read straight from the parameter block, whose
 // fields the instructions take as constant-bank operands (measurably faster
 // for the per-stage bookkeeping at small stages).
-template <int NB, bool kSet>
+// kShort: stage widths are a round's own (a run-time width costs whole stages
+// 1.5%, so launches of long rounds keep the constant).
+template <int NB, bool kSet, bool kShort>
 __global__ void __launch_bounds__(kThreads, 1) k_gemv(const __grid_constant__ MultiArgs a) {
   using CF = Cfg<NB>;
   extern __shared__ __align__(16) uint64_t smem[];
@@ -471,6 +475,13 @@ __global__ void __launch_bounds__(kThreads, 1) k_gemv(const __grid_constant__ Mu
     static_assert(CF::RG <= 8, "round size");
     int np = 0, nst_total = 0;
     int64_t uu = u;
+    // Columns per stage (kShort): a round too short to give every warp a whole
+    // stage is shared out evenly.
+    int st = CF::ST;
+    if constexpr (kShort) {
+      const int64_t cols = min(rend, tub + ((u - tub) / tnb + CF::RG) * tnb) - u;
+      if (cols < CF::ST * kWarps) st = max(kMinStage, ((int)cols + kWarps - 1) / kWarps);
+    }
     const int ck = threadIdx.x >> 5, cln = threadIdx.x & 31;
     int64_t cg = 0;
     // Pieces whose row records this thread stages (record words i, i + kThreads).
@@ -490,7 +501,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_gemv(const __grid_constant__ Mu
       if (np == rk0) rg0 = g;
       if (np == rk1) rg1 = g;
       any_cut |= !(ca == 0 && cbk == tnb);
-      nst_total += (cbk - ca + CF::ST - 1) / CF::ST;
+      nst_total += kShort ? (cbk - ca + st - 1) / st : (cbk - ca + CF::ST - 1) / CF::ST;
       ++np;
       uu += cbk - ca;
     }
@@ -522,7 +533,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_gemv(const __grid_constant__ Mu
       }
     }
     __syncthreads();
-    warp_round<NB>(T, a.n, rdn, tabs, sbuf, xbuf, rrec, pcs, pst, np, nst_total, comb, warp, lane);
+    warp_round<NB, kShort>(T, a.n, rdn, tabs, sbuf, xbuf, rrec, pcs, pst, np, nst_total, st, comb, warp, lane);
     if (ck < np) srow[threadIdx.x] = crow;
     __syncthreads();
     // Row sums of the round's pieces (warps added in warp order), every (piece,
@@ -694,42 +705,64 @@ static size_t smem_bytes() {
 
 using FusedKernel = void (*)(MultiArgs);
 
-template <int NB, bool kSet>
+template <int NB, bool kSet, bool kShort>
 static FusedKernel fused_kernel() {
   if constexpr (on_tensor_cores(NB)) return k_gemm<NB, kSet>;
-  else return k_gemv<NB, kSet>;
+  else return k_gemv<NB, kSet, kShort>;
 }
 
 // The fused kernel's dynamic shared-memory limit is a per-device attribute:
 // set once per device (any host thread), and set again if a launch reports an
 // invalid configuration (the device's context may have been reset since).
-template <int NB, bool kSet>
+template <int NB, bool kSet, bool kShort>
 static DeviceOnce &smem_once() {
   static DeviceOnce once;
   return once;
 }
 
-template <int NB, bool kSet>
+template <int NB, bool kSet, bool kShort>
 static cudaError_t set_smem_limit(int dev) {
-  return (cudaError_t)smem_once<NB, kSet>().run(dev, [] {
-    return (int)cudaFuncSetAttribute(fused_kernel<NB, kSet>(), cudaFuncAttributeMaxDynamicSharedMemorySize,
+  return (cudaError_t)smem_once<NB, kSet, kShort>().run(dev, [] {
+    return (int)cudaFuncSetAttribute(fused_kernel<NB, kSet, kShort>(), cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      (int)smem_bytes<NB>());
   });
 }
 
-template <int NB, bool kSet>
-static cudaError_t launch_fused(const cudaLaunchConfig_t &cfg, const MultiArgs &a) {
+template <int NB, bool kSet, bool kShort>
+static cudaError_t launch_fused_as(const cudaLaunchConfig_t &cfg, const MultiArgs &a) {
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
-  if (e == cudaSuccess) e = set_smem_limit<NB, kSet>(dev);
-  if (e == cudaSuccess) e = cudaLaunchKernelEx(&cfg, fused_kernel<NB, kSet>(), a);
+  if (e == cudaSuccess) e = set_smem_limit<NB, kSet, kShort>(dev);
+  if (e == cudaSuccess) e = cudaLaunchKernelEx(&cfg, fused_kernel<NB, kSet, kShort>(), a);
   if (e == cudaErrorInvalidValue) {
     (void)cudaGetLastError();
-    smem_once<NB, kSet>().forget(dev);
-    e = set_smem_limit<NB, kSet>(dev);
-    if (e == cudaSuccess) e = cudaLaunchKernelEx(&cfg, fused_kernel<NB, kSet>(), a);
+    smem_once<NB, kSet, kShort>().forget(dev);
+    e = set_smem_limit<NB, kSet, kShort>(dev);
+    if (e == cudaSuccess) e = cudaLaunchKernelEx(&cfg, fused_kernel<NB, kSet, kShort>(), a);
   }
   return e;
+}
+
+// Launches of short rounds take the kernel that fits the stage width to the
+// round: at full width a round of 27 columns (1024 x 1024 at b1) keeps one warp
+// of twelve busy.  A round wide enough for half the warps gains nothing from
+// more of them, and the narrower stages cost it.  With several tensors some
+// CTAs have a round on each side of a tensor's end, and those finish last:
+// there the line is a whole stage per warp.  For n >= 2 (narrower stages, more
+// to stage per column) it lies at a quarter of the warps.  Measured, full width
+// / fitted, us: b1 1024 x 1024 14.5 / 12.5, 64 x 11008 20.0 / 17.2, 2048 x 2816
+// 16.5 / 16.5, 5120 x 2048 20.4 / 20.6, a d = 1024 layer 28.8 / 24.9; b4 512 x
+// 1024 16.0 / 14.5, 64 x 11008 30.8 / 26.9, 2048 x 1024 16.5 / 16.5, 4096 x 1024
+// 16.6 / 18.6.
+template <int NB, bool kSet>
+static cudaError_t launch_fused(const cudaLaunchConfig_t &cfg, const MultiArgs &a, int64_t units) {
+  if constexpr (on_tensor_cores(NB)) {
+    return launch_fused_as<NB, kSet, false>(cfg, a);
+  } else {
+    const int64_t full = (int64_t)a.ctas * (Cfg<NB>::ST * kWarps);
+    const int64_t line = NB > 1 ? full / 4 : a.nt > 1 ? full : full / 2;
+    return units < line ? launch_fused_as<NB, kSet, true>(cfg, a) : launch_fused_as<NB, kSet, false>(cfg, a);
+  }
 }
 
 // Cost-balanced ranges of the units of all tensors, one per CTA.  A group's
@@ -881,7 +914,7 @@ static seedq_status launch(const seedq_layer *const *layers, int nt, const uint1
       attr[0].val.programmaticStreamSerializationAllowed = 1;
       cfg.attrs = attr;
       cfg.numAttrs = 1;
-      e = launch_fused<NB, false>(cfg, *a);
+      e = launch_fused<NB, false>(cfg, *a, a->cta_begin[a->ctas]);
     }
     if (e != cudaSuccess) rc = cuda_fail(e);
   }
@@ -919,6 +952,7 @@ struct seedq_layer_set {
   int64_t *d_cta[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};  // per batch template
   int ctas[5] = {0, 0, 0, 0, 0};
   int64_t maxC = 0;
+  int64_t units = 0;                     // (row group, column) units of all tensors
 };
 
 namespace seedq {
@@ -954,7 +988,7 @@ static seedq_status launch_set(const seedq_layer_set *S, const uint16_t *X, int 
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    e = launch_fused<NB, true>(cfg, a);
+    e = launch_fused<NB, true>(cfg, a, S->units);
   }
   return e == cudaSuccess ? SEEDQ_OK : cuda_fail(e);
 }
@@ -992,6 +1026,7 @@ seedq_status seedq_layer_set_create(const seedq_layer *const *layers, int32_t co
     S->cpre[i + 1] = S->cpre[i] + layers[i]->args.C;
     S->rpre[i + 1] = S->rpre[i] + layers[i]->args.R;
     if (layers[i]->args.C > S->maxC) S->maxC = layers[i]->args.C;
+    S->units += (layers[i]->args.R + 31) / 32 * layers[i]->args.nb;
   }
   S->cols = S->cpre[count];
   S->rows = S->rpre[count];
