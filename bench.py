@@ -508,8 +508,8 @@ def encode_inputs(S, k, nblocks):
 
 
 def encode_flops_per_seed(k):
-    """fp64 operations of one seed's fit as the search performs them: the
-    right-hand side (8 products and 8 sums per coefficient), the elimination
+    """fp64 operations of one seed's fit as the exhaustive kernels perform them
+    (the smallest calls; the others are screened): the right-hand side (8 products and 8 sums per coefficient), the elimination
     and back substitution (one division, product and difference per entry
     touched), two exponent probes (one product per mantissa), the mantissas,
     and the error (a product by the exponent, a difference, a square and a
@@ -652,9 +652,14 @@ def encode_arm(args):
     e2e_ms = dist_max(statistics.mean(e2e))
 
     nseeds = (1 << S) - 1
-    flops = encode_flops_per_seed(k) * nseeds * nb
+    screened = S > 8 or k > 3 or nb > 2048  # the library's rule
+    # Screened search: every (block, seed) pair's products of depth 8 with the
+    # seed's k (span) or 8 - k (complement) vectors, on the tensor cores.
+    per_seed = 16 * (k if k <= 3 else 8 - k) if screened else encode_flops_per_seed(k)
+    flops = per_seed * nseeds * nb
     achieved = flops / (step_ms * 1e-3) / 1e12
-    peak = fp64_peak_tflops(Q, stream)
+    pk = measured_peaks()
+    peak = (pk["bf16_tflops"] if pk else 1900.0) if screened else fp64_peak_tflops(Q, stream)
     line = {
         "metric": ENC_METRIC, "value": world * nb / (step_ms * 1e-3), "unit": "blocks/s",
         "n_gpus": world, "steps": args.steps, "warmup": max(args.warmup, 3), "ms_per_step": step_ms,
@@ -668,12 +673,15 @@ def encode_arm(args):
         "e2e": {"value": world * nb / (e2e_ms * 1e-3), "unit": "blocks/s",
                 "h2d_bytes_per_step": w.nbytes,
                 "d2h_bytes_per_step": sum(x.numel() * x.element_size() for x in (seed, E, t, err))},
-        "gpu_launches": args.steps,
-        "roofline": {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
-                     "frac": achieved / peak, "traffic": None, "kernel": "k_encode_list",
-                     "peak_basis": "measured: fp64 FMA loop (seedq_fp64_fma_probe, 8 independent "
-                                   "chains per thread, best of 5 launches, CUDA events); nominal 1.25",
-                     "flops_per_seed": encode_flops_per_seed(k)},
+        "gpu_launches": args.steps * (3 if screened else 1),
+        "roofline": {"bound": "tensor" if screened else "alu", "achieved": achieved, "peak": peak,
+                     "unit": "TFLOP/s", "frac": achieved / peak, "traffic": None,
+                     "kernel": "k_screen" if screened else "k_encode_list",
+                     "peak_basis": ("MEASURED_PEAKS.json bf16_tflops (measured)" if pk else "fallback")
+                     if screened else
+                     "measured: fp64 FMA loop (seedq_fp64_fma_probe, 8 independent "
+                     "chains per thread, best of 5 launches, CUDA events); nominal 1.25",
+                     "flops_per_seed": per_seed},
     }
     if rank == 0 and not args.no_cpu_baseline:
         run, n = encode_oracle_sample(S, k, w, 10.0, cpu_cores())
@@ -920,8 +928,8 @@ def allocate_arm(args):
     for _ in range(max(args.warmup, 3)):
         got = step()
     assert list(got[0]) == d["theta"] and [int(x) for x in got[3]] == d["tie_count"]
-    # Latency floor of one bisection step: a launch, an 8-byte read-back and a
-    # host synchronization (the allocator needs the count before the next step).
+    # Latency of a bisection step driven from the host: a launch, an 8-byte
+    # read-back and a synchronization (the device runs the steps without them).
     one = torch.zeros(1, dtype=torch.int16, device="cuda")
     host = torch.zeros(1, dtype=torch.int16, pin_memory=True)
     for _ in range(20):
@@ -947,6 +955,13 @@ def allocate_arm(args):
     # Evaluations: the floor's and the multiplier's bisections over 64-bit
     # patterns, plus the two end points, the tied group and the demotion counts.
     evals = 64 + 64 + 5
+    # Launches: two rankings, the factors, two searches in rounds of up to 31
+    # points (as many as keep a round near 2^16 row searches), group and tail.
+    rows, probes = sum(R if rho is not None else 1 for R, C, a, rho in factors), 31
+    while probes > 1 and rows * probes > 1 << 16:
+        probes //= 2
+    per_round = (probes + 1).bit_length() - 1
+    launches = 3 + 2 * ((63 + per_round - 1) // per_round + 1) + 2
     line = {
         "metric": ALLOC_METRIC, "value": world / step_s, "unit": "allocations/s",
         "n_gpus": world, "steps": args.steps, "warmup": max(args.warmup, 3),
@@ -954,18 +969,18 @@ def allocate_arm(args):
         "vs_baseline": None, "dtype": "f64", "data": "synthetic",
         "config": {"workload": f"{w.name}: {w.description}", "tensors": len(w.tensors),
                    "timing": "host wall clock around the synchronous call (it includes the "
-                             "factor upload and kernels and ~130 dependent evaluations)"},
+                             "factor upload and kernels and the searches' dependent rounds)"},
         "clocks": clk,
         "e2e": {"value": world / step_s, "unit": "allocations/s",
                 "h2d_bytes_per_step": sum(4 * (C + (R if rho is not None else 0))
                                           for R, C, a, rho in factors),
-                "d2h_bytes_per_step": 8 * (1 + len(factors) + 9) * evals},
-        "gpu_launches": args.steps * (3 * len(factors) + evals),
+                "d2h_bytes_per_step": 8 * (2 * len(factors) + 47)},
+        "gpu_launches": args.steps * launches,
         "roofline": {"bound": "latency", "achieved": evals / step_s, "peak": 1.0 / rt,
                      "unit": "dependent evaluations/s", "frac": rt * evals / step_s,
-                     "traffic": None, "kernel": "k_alloc_eval (one per bisection step)",
+                     "traffic": None, "kernel": "k_alloc_round (several points a launch)",
                      "peak_basis": "measured launch + 8-byte read-back + synchronize round trip "
-                                   f"({rt * 1e6:.1f} us)"},
+                                   f"({rt * 1e6:.1f} us); above 1: the searches stay on the device"},
     }
     if rank == 0 and not args.no_cpu_baseline:
         t = allocate_oracle(args.workload, w, d)

@@ -25,7 +25,7 @@
 // the order of evaluation.
 //
 // What bounds it: at (16, 3) the latency of the product chain (16 warps per
-// SM; issue active 41% of cycles, tensor pipe 31%) ahead of the fp64 pipe (the
+// SM; issue active 44% of cycles, tensor pipe 45%) ahead of the fp64 pipe (the
 // evaluations, 28 a block); at K >= 5 the evaluations (200 to 1000 a block).
 // Measured on one GB300 against the exhaustive kernels (every pair solved):
 // 32768 blocks at (16, 3) 446 -> 0.84 ms (39 M blocks/s; the 2.1 G pairs'

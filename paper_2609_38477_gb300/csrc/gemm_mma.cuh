@@ -34,8 +34,8 @@
 // partial sums in scratch, and the CTA that arrives last adds them in CTA
 // order.
 //
-// Bound by issue (52% of cycles, 125 instructions per 32 blocks at k = 2, 150
-// at k = 3; ALU 45%, tensor pipe 14% to 19%): the reconstruction, the split
+// Bound by issue (46% to 52% of cycles, 125 instructions per 32 blocks at k = 2,
+// 150 at k = 3; ALU 40% to 45%, tensor pipe 14% to 19%): the reconstruction, the split
 // (8 logic and 8 packed fp32 instructions a block) and rows that change rung at
 // different columns.  The FMA kernel issued 253 at b16, 96 of them products and
 // activation loads.  Measured on one GB300 against it: a 7B layer at 4.0 bits,
