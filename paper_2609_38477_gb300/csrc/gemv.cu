@@ -818,7 +818,7 @@ static void partition(const seedq_layer *const *layers, int nt, int n, int64_t *
         double acc = g0;
         int col = nb, clo = 0;
         if (gs > 1) {  // by the superblock's work profile
-          const float *prof = L->h_prof + g * 2 * (kProfile + 1);
+          const float *prof = L->h_prof + g * kProfileFloats;
           auto at = [&](int i) { return g0 + kCostK * prof[kProfile + 1 + i] + cb * prof[i]; };
           int i = 1;
           while (i < kProfile && at(i) <= lt) ++i;

@@ -551,7 +551,7 @@ static seedq_status build_costs(seedq_layer *L, cudaStream_t st) {
   L->h_mp = (double *)malloc(sizeof(double) * (G + 1));
   L->h_mk = (double *)malloc(sizeof(double) * (G + 1));
   const int64_t SB = (G + kMmGroups - 1) / kMmGroups;
-  L->h_prof = (float *)calloc((size_t)SB * 2 * (kProfile + 1), sizeof(float));
+  L->h_prof = (float *)calloc((size_t)SB * kProfileFloats, sizeof(float));
   L->h_repbk = (int32_t *)malloc(sizeof(int32_t) * G * Jm1);
   const int nst = (nb + kCostStage - 1) / kCostStage;
   uint8_t *mixed = (uint8_t *)malloc(nst);
@@ -569,8 +569,7 @@ static seedq_status build_costs(seedq_layer *L, cudaStream_t st) {
     L->h_mp[0] = 0.0;
     L->h_mk[0] = 0.0;
     const int32_t *rowb[32];
-    int32_t last_bk[kMaxJ] = {0};
-    bool last_uniform = false;
+    MmProfile mm(nb, J, L->k);
     for (int64_t g = 0; g < G; ++g) {
       int nr = 0;
       for (int i = 0; i < 32 && g * 32 + i < R; ++i) rowb[nr++] = brk + (int64_t)rowperm[g * 32 + i] * Jm1;
@@ -585,59 +584,8 @@ static seedq_status build_costs(seedq_layer *L, cudaStream_t st) {
         K += (double)L->k[j] * (hi - lo);
         lo = hi;
       }
-      // The tensor-core kernel passes, for each set of sixteen rows, over
-      // every column one of them has at a rung; a pass of the group's 32 rows
-      // over a stage costs about five columns more (fitted to per-CTA times).
       double mP = 0.0, mK = 0.0;
-      float *prof = L->h_prof + (g / kMmGroups) * 2 * (kProfile + 1);
-      constexpr double kPass = 5.0;
-      auto add = [&](int from, int to, double wp, double wk) {
-        mP += wp * (to - from);
-        mK += wk * (to - from);
-        for (int i = 1; i <= kProfile; ++i) {
-          const int c = (int)((int64_t)nb * i / kProfile), n = (c < to ? c : to) - from;
-          if (n <= 0) continue;
-          prof[i] += (float)(wp * n);
-          prof[kProfile + 1 + i] += (float)(wk * n);
-        }
-      };
-      // A group whose rows all have the last one's breakpoints repeats its
-      // profile (tensors without a row factor: every group).
-      bool same = g > 0 && g % kMmGroups != 0;
-      for (int i = 0; i < nr && same; ++i)
-        for (int j = 0; j < J - 1; ++j) same = same && rowb[i][j] == last_bk[j];
-      if (L->max_batch <= 4) {
-        // (never launched)
-      } else if (same && last_uniform) {
-        mP = L->h_mp[g] - L->h_mp[g - 1];
-        mK = L->h_mk[g] - L->h_mk[g - 1];
-        const float f = (float)(g % kMmGroups + 1) / (float)(g % kMmGroups);
-        for (int i = 0; i < 2 * (kProfile + 1); ++i) prof[i] *= f;
-      } else {
-        for (int j = 0; j < J; ++j) {
-          int from32 = nb, to32 = 0;
-          for (int s0 = 0; s0 < nr; s0 += 16) {
-            int from = nb, to = 0;
-            for (int i = s0; i < nr && i < s0 + 16; ++i) {
-              const int a = (j > 0) ? rowb[i][j - 1] : 0, z = (j < J - 1) ? rowb[i][j] : nb;
-              if (a < z) {
-                from = a < from ? a : from;
-                to = z > to ? z : to;
-              }
-            }
-            if (from < to) add(from, to, 0.5, 0.5 * L->k[j]);
-            from32 = from < from32 ? from : from32;
-            to32 = to > to32 ? to : to32;
-          }
-          // One pass per stage it touches: len / 24 of them, and one more.
-          if (from32 < to32) add(from32, to32, kPass / kCostStage + kPass / (to32 - from32), 0.0);
-        }
-        last_uniform = nr == 32;
-        for (int j = 0; j < J - 1; ++j) {
-          last_bk[j] = rowb[0][j];
-          for (int i = 1; i < nr; ++i) last_uniform = last_uniform && rowb[i][j] == rowb[0][j];
-        }
-      }
+      if (L->max_batch > 4) mm.add(rowb, nr, L->h_prof + (g / kMmGroups) * kProfileFloats, mP, mK);
       L->h_mp[g + 1] = L->h_mp[g] + mP;
       L->h_mk[g + 1] = L->h_mk[g] + mK;
       // Stages where the rows' breakpoints differ: replace the first row's

@@ -6,10 +6,10 @@
 
 #include "../../include/seedq.h"
 #include "f32x2.cuh"
+#include "mm_profile.h"
 
 namespace seedq {
 
-constexpr int kMaxJ = 9;         // hull rungs (App. B.3: four to eight on the paper's grids)
 constexpr int kMaxOutliers = 16; // FP16 outlier columns (Sec. 3.5 stores four)
 constexpr int kMaxBatch = 16;    // decode batch of seedq_gemm_small_batch
 constexpr int kMaxCols = 65536;
@@ -69,11 +69,6 @@ constexpr double kCostK = 1.0;
 inline double cost_block(int n) {
   return n <= 1 ? 3.7 : n <= 2 ? 5.3 : n <= 4 ? 8.4 : 8.0;
 }
-// Stage width (blocks) the work profile assumes.
-constexpr int kCostStage = 24;
-// Columns at which a superblock's work profile is kept.
-constexpr int kProfile = 16;
-constexpr int kMmGroups = 4;  // row groups of a superblock
 // Floats of one CTA's partial sums of a cut group (k_gemv: 32 rows) or
 // superblock (k_gemm: 128 rows) at batch template nb.
 inline int slot_floats(int nb) { return nb > 4 ? 128 * nb : 32 * kMaxBatch; }
