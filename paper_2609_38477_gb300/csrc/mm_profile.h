@@ -34,6 +34,10 @@ class MmProfile {
       for (int i = 1; i < nr && have_; ++i) have_ = equal(rowb[i], rowb[0]);
       for (int j = 0; j < J_ - 1; ++j) bk_[j] = rowb[0][j];
     }
+    repeat(prof, P, K);
+  }
+  // The same for a group known to have the breakpoints of the last one.
+  void repeat(float *prof, double &P, double &K) const {
     P = P_;
     K = K_;
     for (int i = 0; i < kProfileFloats; ++i) prof[i] += own_[i];
