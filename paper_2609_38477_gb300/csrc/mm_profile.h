@@ -10,6 +10,11 @@ constexpr int kMaxJ = 9;        // hull rungs (App. B.3: four to eight on the pa
 constexpr int kCostStage = 24;  // stage width (blocks) the profiles assume
 constexpr int kProfile = 16;    // columns at which a superblock's profile is kept
 constexpr int kMmGroups = 4;    // row groups of a superblock
+// Time of a superblock's column that an idle group saves none of, as a share of
+// a busy group's.  Measured at 0 / 0.3 / 0.5 / 0.65 / 0.8 / 0.95, b8: 5000 x 5008
+// (its last superblock holds 8 rows) 103 / 60 / 48 / 46.6 / 45.5 / 46.5 us, 38408
+// x 5008 252 / 227 / 213 / 203 / 197 / 197; 5120 x 5008 45.4.
+constexpr double kIdleGroup = 0.8;
 constexpr int kProfileFloats = 2 * (kProfile + 1);
 
 // For each set of sixteen rows the kernel passes over every column one of them
@@ -41,6 +46,16 @@ class MmProfile {
     P = P_;
     K = K_;
     for (int i = 0; i < kProfileFloats; ++i) prof[i] += own_[i];
+  }
+
+  // Makes a superblock of fewer groups cost what it takes: its columns pass
+  // through a CTA hardly faster than a whole one's, the warps of the missing
+  // groups idle.  P and K: its groups' sums.
+  static void partial(int groups, float *prof, double &P, double &K) {
+    const double f = 1.0 + kIdleGroup * (kMmGroups - groups) / groups;
+    P *= f;
+    K *= f;
+    for (int i = 0; i < kProfileFloats; ++i) prof[i] = (float)(prof[i] * f);
   }
 
  private:

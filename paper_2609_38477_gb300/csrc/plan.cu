@@ -642,6 +642,13 @@ static seedq_status build_costs(seedq_layer *L, cudaStream_t st) {
       }
       L->h_mp[g + 1] = L->h_mp[g] + mP;
       L->h_mk[g + 1] = L->h_mk[g] + mK;
+      if (g == G - 1 && G % kMmGroups != 0 && L->max_batch > 4) {
+        const int64_t g0 = g / kMmGroups * kMmGroups;
+        double sP = L->h_mp[G] - L->h_mp[g0], sK = L->h_mk[G] - L->h_mk[g0];
+        MmProfile::partial((int)(G - g0), prof, sP, sK);
+        L->h_mp[G] = L->h_mp[g0] + sP;
+        L->h_mk[G] = L->h_mk[g0] + sK;
+      }
       L->h_gp[g + 1] = L->h_gp[g] + P;
       L->h_gk[g + 1] = L->h_gk[g] + K;
     }

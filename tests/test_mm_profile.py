@@ -71,3 +71,38 @@ def test_superblock_profile_is_the_sum_of_its_groups(tmp_path):
     assert r.returncode == 0, r.stderr
     r = subprocess.run([str(exe)], capture_output=True, text=True, timeout=60)
     assert r.returncode == 0 and r.stdout.strip() == "ok", r.stdout + r.stderr
+
+
+PARTIAL = r"""
+#include "mm_profile.h"
+#include <cmath>
+#include <cstdio>
+using namespace seedq;
+
+int main() {
+  for (int groups = 1; groups <= kMmGroups; ++groups) {
+    float prof[kProfileFloats];
+    for (int i = 0; i < kProfileFloats; ++i) prof[i] = (float)(i * groups);
+    double P = 10.0 * groups, K = 30.0 * groups;
+    MmProfile::partial(groups, prof, P, K);
+    // Between its groups' own cost and a whole superblock's; the profile in step.
+    if (P < 10.0 * groups || P > 10.0 * kMmGroups + 1e-9 || std::fabs(K - 3 * P) > 1e-9) return 1;
+    for (int i = 0; i < kProfileFloats; ++i)
+      if (std::fabs(prof[i] - i * P / 10.0) > 1e-4 * (1 + prof[i])) return 2;
+  }
+  std::printf("ok\n");
+  return 0;
+}
+"""
+
+
+@pytest.mark.skipif(shutil.which("g++") is None, reason="needs g++")
+def test_partial_superblock(tmp_path):
+    src = tmp_path / "partial.cpp"
+    src.write_text(PARTIAL)
+    exe = tmp_path / "partial"
+    r = subprocess.run(["g++", "-std=c++17", "-O1", "-I", CSRC, str(src), "-o", str(exe)],
+                       capture_output=True, text=True)
+    assert r.returncode == 0, r.stderr
+    r = subprocess.run([str(exe)], capture_output=True, text=True, timeout=60)
+    assert r.returncode == 0 and r.stdout.strip() == "ok", r.stdout + r.stderr
