@@ -32,14 +32,14 @@
 // pre-kernel) are copied once for all four groups.  Partial sums of the three
 // column parts are added in part order; superblocks cut between CTAs leave
 // partial sums in scratch, and the CTA that arrives last adds them in CTA
-// order.
+// order (up to 80 of them, four outputs a thread and eight loads in flight).
 //
 // Bound by issue (46% to 52% of cycles, 125 instructions per 32 blocks at k = 2,
 // 150 at k = 3; ALU 40% to 45%, tensor pipe 14% to 19%): the reconstruction, the split
 // (8 logic and 8 packed fp32 instructions a block) and rows that change rung at
 // different columns.  The FMA kernel issued 253 at b16, 96 of them products and
 // activation loads.  Measured on one GB300 against it: a 7B layer at 4.0 bits,
-// b16 381 -> 268 us; two 70B layers at 3.0 bits, b8 1932 -> 1505 us.  Tried:
+// b16 381 -> 260 us; two 70B layers at 3.0 bits, b8 1935 -> 1530 us.  Tried:
 // masked and unmasked segments of a pass apart (3% to 5% slower), eight warps
 // with 242 registers (3% faster at b16, 8% slower at b8), sixteen warps with
 // 128 (14% slower), the 11-bit and 10-bit parts in separate sums (equal).
@@ -347,6 +347,104 @@ struct MmSum {
   __device__ __forceinline__ float value() const { return isfinite(s) ? __fadd_rn(s, e) : s; }
 };
 
+// T, and where it is a kernel parameter its copy in the CTA's shared memory, for
+// code out of line: taken by address there it costs the main loop its constant
+// operands (a 7B layer at b8 235 -> 239 us).
+template <bool kSet>
+__device__ __forceinline__ const TensorArgs &mm_shared(const TensorArgs &T, TensorArgs &sT) {
+  if constexpr (kSet) return T;
+  __syncthreads();
+  if (threadIdx.x == 0) sT = T;
+  __syncthreads();
+  return sT;
+}
+
+// Output i (row, batch entry) of a superblock from the column parts' sums.
+template <int NB>
+__device__ __forceinline__ float mm_parts(const float *comb, int i) {
+  MmSum sum;
+#pragma unroll
+  for (int k = 0; k < kMmParts; ++k) sum.add(comb[k * kMmRows * NB + i]);
+  return sum.value();
+}
+
+// y of a superblock that one CTA has whole.
+template <int NB, bool kSet>
+__device__ __forceinline__ void mm_write(const TensorArgs &T, int n, const uint16_t *X, float *Y, int64_t sb, float *comb,
+                                         TensorArgs &sT) {
+  const LayerArgs &p = T.p;
+  const int64_t row0 = sb * kMmRows;
+  uint32_t bad = 0u;
+  for (int i = threadIdx.x; i < kMmRows * NB; i += kMmThreads) {
+    const int row = i / NB, b = i % NB;
+    if (row0 + row >= p.R || b >= n) continue;
+    const int64_t rr = __ldg(p.rowperm + row0 + row);
+    const float v = mm_parts<NB>(comb, i);
+    if (!isfinite(v)) bad |= 1u << b;
+    Y[(int64_t)b * p.R + rr] = v + outlier_term(p, X, rr, b);
+  }
+  if (__syncthreads_or(bad != 0u)) mm_nonfinite<NB>(mm_shared<kSet>(T, sT), X, Y, sb, bad, reinterpret_cast<uint32_t *>(comb));
+}
+
+// The CTA's partial sums of a cut superblock (tensor T, superblock sb) are in
+// its slots: counts the CTA's arrival, and where it is the last, adds all of
+// them in CTA order and writes y.  No CTA waits for another.
+template <int NB, bool kSet>
+__device__ __forceinline__ void mm_finish(const TensorArgs &T, const int64_t *cb, int ctas, int n, const uint16_t *X,
+                                          float *Y, int64_t sb, uint32_t *list, TensorArgs &sT) {
+  __shared__ int s_last;
+  const LayerArgs &p = T.p;
+  const int64_t gu = T.ubegin_mm + sb * p.nb;
+  const int cf = cta_of(cb, ctas, gu), cl = cta_of(cb, ctas, gu + p.nb - 1);
+  __syncthreads();  // (the last call's s_last)
+  if (threadIdx.x == 0) s_last = atomicAdd(p.counters + sb, 1) == cl - cf;
+  __syncthreads();
+  if (!s_last) return;
+  __threadfence();
+  // The first CTA's range may start before this superblock, the others' start in
+  // it.  Four neighbouring outputs per thread, kAhead CTAs' sums in flight.
+  constexpr int kAhead = 8, kPiece = kMmRows * NB / 4;
+  const float4 *slots = reinterpret_cast<const float4 *>(p.slots);
+  const float4 *first = slots + ((int64_t)cf * 2 + (cb[cf] >= gu ? 0 : 1)) * kPiece;
+  const float4 *rest = slots + (int64_t)(cf + 1) * 2 * kPiece;
+  const int others = cl - cf;
+  uint32_t bad = 0u;
+  for (int i = threadIdx.x; i < kPiece; i += kMmThreads) {
+    const int row = i / (NB / 4), b0 = i % (NB / 4) * 4;
+    const int64_t pos = sb * kMmRows + row;
+    if (pos >= p.R) continue;
+    MmSum sum[4];
+    auto add = [&](const float4 &v) {
+      sum[0].add(v.x);
+      sum[1].add(v.y);
+      sum[2].add(v.z);
+      sum[3].add(v.w);
+    };
+    add(__ldcg(first + i));
+    const float4 *at = rest + i;
+    int c = 0;
+    for (; c + kAhead <= others; c += kAhead, at += 2 * kAhead * kPiece) {
+      float4 v[kAhead];
+#pragma unroll
+      for (int k = 0; k < kAhead; ++k) v[k] = __ldcg(at + 2 * k * kPiece);
+#pragma unroll
+      for (int k = 0; k < kAhead; ++k) add(v[k]);
+    }
+    for (; c < others; ++c, at += 2 * kPiece) add(__ldcg(at));
+    const int64_t rr = __ldg(p.rowperm + pos);
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      const int b = b0 + e;
+      if (b >= n) continue;
+      const float v = sum[e].value();
+      if (!isfinite(v)) bad |= 1u << b;
+      Y[(int64_t)b * p.R + rr] = v + outlier_term(p, X, rr, b);
+    }
+  }
+  if (__syncthreads_or(bad != 0u)) mm_nonfinite<NB>(mm_shared<kSet>(T, sT), X, Y, sb, bad, list);
+  if (threadIdx.x == 0) p.counters[sb] = 0;
+}
+
 template <int NB, bool kSet>
 __global__ void __launch_bounds__(kMmThreads, 1) k_gemm(const __grid_constant__ MultiArgs a) {
   using CF = MmCfg<NB>;
@@ -360,7 +458,8 @@ __global__ void __launch_bounds__(kMmThreads, 1) k_gemm(const __grid_constant__ 
   float *comb = reinterpret_cast<float *>(xbuf);  // after a piece's last window
   __shared__ TensorArgs sT;
   __shared__ uint4 rdn[kMaxJ * RungDn<2>::kEntry];
-  __shared__ int sflag[2];
+  __shared__ int cut_ti[2];
+  __shared__ int64_t cut_sb[2];
   {
     // The jump tables depend only on S, so any tensor's copy serves all.
     const uint4 *src = reinterpret_cast<const uint4 *>((kSet ? a.tens : a.t)[0].p.tables);
@@ -383,8 +482,8 @@ __global__ void __launch_bounds__(kMmThreads, 1) k_gemm(const __grid_constant__ 
     }
     ti = lo;
   }
-  int cut_ti[2] = {-1, -1};  // superblocks cut where the range starts and ends
-  int64_t cut_sb[2] = {0, 0};
+  // Superblocks cut where the range starts and ends (tensor -1: none).
+  if (threadIdx.x < 2) cut_ti[threadIdx.x] = -1;
   for (int64_t u = u0; u < u1;) {
     while (ti + 1 < a.nt && tens[ti + 1].ubegin_mm <= u) ++ti;
     __syncthreads();  // the last piece is done with sT, rdn and the buffers
@@ -397,8 +496,6 @@ __global__ void __launch_bounds__(kMmThreads, 1) k_gemm(const __grid_constant__ 
     __syncthreads();
     const TensorArgs &T = kSet ? sT : a.t[ti];
     const LayerArgs &p = T.p;
-    const uint16_t *X = kSet ? a.Xall + (int64_t)a.n * T.cpre : T.x;
-    float *Y = kSet ? a.Yall + (int64_t)a.n * T.rpre : T.y;
     const int nb = p.nb, J = p.J;
     const int64_t lu = u - T.ubegin_mm, tend = (ti + 1 < a.nt) ? tens[ti + 1].ubegin_mm : cb[a.ctas];
     const int64_t sb = lu / nb;
@@ -564,65 +661,29 @@ __global__ void __launch_bounds__(kMmThreads, 1) k_gemm(const __grid_constant__ 
     __syncthreads();
     const bool full = ca == 0 && cbk == nb;
     const int side = u == u0 ? 0 : 1;
-    const int64_t row0 = sb * kMmRows;
-    uint32_t bad = 0u;
-    for (int i = threadIdx.x; i < kMmRows * NB; i += kMmThreads) {
-      const int row = i / NB, b = i % NB;
-      MmSum sum;
-#pragma unroll
-      for (int k = 0; k < kMmParts; ++k) sum.add(comb[(k * kMmRows + row) * NB + b]);
-      if (!full) {
-        p.slots[((int64_t)cta * 2 + side) * kMmRows * NB + i] = sum.value();
-      } else if (row0 + row < p.R && b < a.n) {
-        const int64_t rr = __ldg(p.rowperm + row0 + row);
-        const float v = sum.value();
-        if (!isfinite(v)) bad |= 1u << b;
-        Y[(int64_t)b * p.R + rr] = v + outlier_term(p, X, rr, b);
+    if (full) {
+      mm_write<NB, kSet>(T, a.n, kSet ? a.Xall + (int64_t)a.n * T.cpre : T.x, kSet ? a.Yall + (int64_t)a.n * T.rpre : T.y,
+                   sb, comb, sT);
+    } else {
+      float *slot = p.slots + ((int64_t)cta * 2 + side) * kMmRows * NB;
+      for (int i = threadIdx.x; i < kMmRows * NB; i += kMmThreads) slot[i] = mm_parts<NB>(comb, i);
+      if (threadIdx.x == 0) {
+        cut_ti[side] = ti;
+        cut_sb[side] = sb;
       }
-    }
-    if (full && __syncthreads_or(bad != 0u)) mm_nonfinite<NB>(T, X, Y, sb, bad, reinterpret_cast<uint32_t *>(comb));
-    if (!full) {
-      cut_ti[side] = ti;
-      cut_sb[side] = sb;
     }
     u += cbk - ca;
   }
-  if (cut_ti[0] < 0 && cut_ti[1] < 0) return;
-  // Each CTA publishes its partial sums of a cut superblock and counts its
-  // arrival; the CTA that arrives last adds them in CTA order and writes y.
-  // No CTA waits for another.
   __threadfence();
   __syncthreads();
 #pragma unroll 1
   for (int side = 0; side < 2; ++side) {
-    if (cut_ti[side] < 0) continue;
-    const TensorArgs &T = tens[cut_ti[side]];
-    const LayerArgs &p = T.p;
-    const int64_t sb = cut_sb[side], gu = T.ubegin_mm + sb * p.nb;
-    const int cf = cta_of(cb, a.ctas, gu), cl = cta_of(cb, a.ctas, gu + p.nb - 1);
-    if (threadIdx.x == 0) sflag[side] = atomicAdd(p.counters + sb, 1) == cl - cf;
-    __syncthreads();
-    if (!sflag[side]) continue;
-    __threadfence();
-    const uint16_t *X = kSet ? a.Xall + (int64_t)a.n * T.cpre : T.x;
-    float *Y = kSet ? a.Yall + (int64_t)a.n * T.rpre : T.y;
-    uint32_t bad = 0u;
-    for (int i = threadIdx.x; i < kMmRows * NB; i += kMmThreads) {
-      const int row = i / NB, b = i % NB;
-      const int64_t pos = sb * kMmRows + row;
-      if (pos >= p.R || b >= a.n) continue;
-      MmSum sum;
-      for (int c2 = cf; c2 <= cl; ++c2) {
-        const int s2 = (cb[c2] >= gu) ? 0 : 1;  // the CTA's range starts in this superblock
-        sum.add(__ldcg(p.slots + ((int64_t)c2 * 2 + s2) * kMmRows * NB + i));
-      }
-      const int64_t rr = __ldg(p.rowperm + pos);
-      const float v = sum.value();
-      if (!isfinite(v)) bad |= 1u << b;
-      Y[(int64_t)b * p.R + rr] = v + outlier_term(p, X, rr, b);
-    }
-    if (__syncthreads_or(bad != 0u)) mm_nonfinite<NB>(T, X, Y, sb, bad, reinterpret_cast<uint32_t *>(comb));
-    if (threadIdx.x == 0) p.counters[sb] = 0;
+    const int ci = cut_ti[side];
+    if (ci < 0) continue;
+    const TensorArgs &T = tens[ci];
+    mm_finish<NB, kSet>(T, cb, a.ctas, a.n, kSet ? a.Xall + (int64_t)a.n * T.cpre : T.x,
+                  kSet ? a.Yall + (int64_t)a.n * T.rpre : T.y, cut_sb[side],
+                  reinterpret_cast<uint32_t *>(comb), sT);
   }
 }
 

@@ -89,9 +89,11 @@ struct MultiArgs {
 
 // Batch templates of up to four run on the FMA pipes (k_gemv), larger ones on
 // the tensor cores (k_gemm).  Measured, k_gemv / k_gemm: a 7B layer at 4.0 bits
-// b4 182 / 232 us, b8 261 / 233, b16 381 / 268; at 3.0 bits b4 166 / 205, b8 265
-// / 217, b16 397 / 250; 1024 x 1024 b8 28 / 19, b16 48 / 39; 256 x 256 b8 35 /
-// 19; 1997 x 2072 b8 31 / 29, b16 48 / 38; 11008 x 128 b16 47 / 31.
+// b8 265 / 238 us, b16 395 / 260; at 3.0 bits b8 246 / 207, b16 367 / 237; a d =
+// 1024 layer b8 38 / 33, b16 54 / 36; 1024 x 1040 b8 27 / 17, b16 47 / 19; 128 x
+// 1040 29 / 16, 52 / 19; 11008 x 128 32 / 17, 46 / 19; 5000 x 5008 52 / 43, 74 /
+// 50.  Of 600 sizes, rates and row factors none was slower.  At b4 (with the cuts
+// of then): a 7B layer 182 / 232, at 3.0 bits 166 / 205.
 __host__ __device__ constexpr bool on_tensor_cores(int NB) { return NB >= 8; }
 
 __host__ __device__ inline int batch_template(int n) {
@@ -765,6 +767,20 @@ static cudaError_t launch_fused(const cudaLaunchConfig_t &cfg, const MultiArgs &
   }
 }
 
+// How the tensor-core launches are cut.  A CTA's fixed cost is about 45 columns
+// of a superblock, once more for a second superblock in its range, and whoever
+// finishes a cut superblock adds all its CTAs' partial sums.  So a CTA gets at
+// least kMmLeast columns, unless that leaves fewer than kMmPer CTAs per
+// superblock, and a cut near a superblock's end moves there: nearer than half a
+// CTA's share while that is below 2 kMmSnap columns, else than kMmSnap.
+// Measured, b8, without these rules (and the sums of a cut superblock added one
+// output at a time) / with them: 128 x 1040 35 / 16 us, 256 x 5008 46 / 21, 640 x
+// 5008 37 / 21, 1600 x 1040 29 / 18, a d = 1024 layer 40 / 33.  At least 8 or 18
+// columns, 16 or 32 CTAs: up to 2% slower.  Moves of 20 columns for all: the d =
+// 1024 layer 38.8; of 40 for all: a d = 2048 layer 69 -> 74.
+constexpr int kMmLeast = 12, kMmPer = 8;
+constexpr double kMmSnap = 20.0;
+
 // Cost-balanced ranges of the units of all tensors, one per CTA.  A group's
 // cost is its modeled time at batch n (block passes and the sum of k over
 // them); inside the group where a range is cut, the first row's rung profile,
@@ -780,17 +796,19 @@ static void partition(const seedq_layer *const *layers, int nt, int n, int64_t *
     const int64_t i = std::min(g * gs, (L->args.R + 31) / 32);
     return gs > 1 ? kCostK * L->h_mk[i] + cb * L->h_mp[i] : kCostK * L->h_gk[i] + cb * L->h_gp[i];
   };
-  int64_t U = 0;
+  int64_t U = 0, sbs = 0;
   double total = 0.0;
   for (int i = 0; i < nt; ++i) {
     const seedq_layer *L = layers[i];
     const int64_t G = groups(L);
     ubegin[i] = U;
+    sbs += G;
     U += G * L->args.nb;
     total += gcost(L, G);
   }
   int ctas = layers[0]->max_ctas;
   if (ctas > kMaxCtas) ctas = kMaxCtas;
+  if (gs > 1) ctas = (int)std::min((int64_t)ctas, std::max(U / kMmLeast, kMmPer * sbs));
   if (U < ctas) ctas = (int)U;
   ctas_out = ctas;
   cta_begin[0] = 0;
@@ -841,6 +859,13 @@ static void partition(const seedq_layer *const *layers, int nt, int n, int64_t *
         if (col < 0) col = 0;
         if (col > nb) col = nb;
         int64_t u = ubegin[ti] + g * nb + col;
+        if (gs > 1) {
+          const double share = total / ctas, snap = kMmSnap * (g1 - g0) / nb;
+          const double near = share < 4.0 * snap ? 0.5 * share : snap;
+          const int64_t e0 = ubegin[ti] + g * nb, e1 = e0 + nb;
+          if (lt - g0 < near && e0 > cta_begin[c - 1]) u = e0;
+          else if (g1 - lt < near && e1 > cta_begin[c - 1]) u = e1;
+        }
         if (u <= cta_begin[c - 1]) u = cta_begin[c - 1] + 1;
         if (u > U - (ctas - c)) u = U - (ctas - c);
         cta_begin[c] = u;
