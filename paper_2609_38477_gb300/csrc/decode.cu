@@ -2,12 +2,15 @@
 //
 // Two kernels.  k_decode_tile builds whole rows in shared memory, where the
 // scatter through the inverse permutation costs bank conflicts, and writes
-// them out as one contiguous bulk copy; it takes every tensor whose row fits.
-// k_decode scatters straight to memory, four bytes to a 32-byte sector: it is
-// left with rows too long for shared memory and outputs that are not 16-byte
-// aligned.
+// them out as one contiguous bulk copy.  k_decode scatters straight to memory,
+// four bytes to a 32-byte sector: it takes the outputs that are small, or of
+// short rows, where that is the faster (tile_is_faster), rows too long for
+// shared memory and outputs that are not 16-byte aligned.
 #include <cuda_fp16.h>
 
+#include <algorithm>
+
+#include "device_once.h"
 #include "seedq_internal.cuh"
 
 namespace seedq {
@@ -89,8 +92,8 @@ __global__ void k_outliers(const __grid_constant__ LayerArgs p, int64_t row0, in
 // eight random words a block, two table lookups, the rung's constants), ahead
 // of the 4 bytes a weight written.  Measured against k_decode on one GB300:
 // 4096 x 11008 with a row factor and four outlier columns 286 -> 72 us (2.8
-// TB/s of weights and stream), 4096 x 4096 94 -> 32, 1024 x 1024 14 -> 10,
-// 512 x 20000 64 -> 29, 33 x 128 10 -> 7; no size in its range was slower.
+// TB/s of weights and stream), 4096 x 4096 94 -> 32, 1024 x 1040 9.2 -> 7.6,
+// 512 x 20000 64 -> 29.
 // On the way: two 512-thread CTAs per SM with barriers around each tile 88 us;
 // the moving warp instead of barriers 80; stream and permutation in shared
 // memory 80; chunks dealt from where the last tile ended 72 (the warps with
@@ -380,6 +383,48 @@ __global__ void __launch_bounds__(kDecThreads + 32, 1)
 }
 static_assert(kDecRows <= 32, "one lane of the storing warp per row record");
 
+// k_decode takes 4.5 us a million weights (the sectors it writes) and, with
+// outliers, a second launch.  k_decode_tile takes 0.6 us more to start and then, for
+// each row an SM gets, 0.07 us and 0.23 us a thousand columns, its first 40 rows
+// 0.13 us more.  Fitted to 500 sizes from 1 x 8 to 60000 x 384 and 8192 x 8192, with
+// and without outliers: at most 9% slower than always direct and 12% (0.9 us) than
+// always tiles.  Measured, direct / tile: 8 x 22400 4.9 / 10.7 us, 4096 x 64 5.2 /
+// 9.1, 8192 x 128 8.4 / 12.3, 4096 x 512 12.9 / 11.1, 1024 x 1040 9.2 / 7.6, 4096 x
+// 11008 278 / 68.
+static bool tile_is_faster(int64_t rows, int64_t C, int sms, bool outliers) {
+  const double weights = (double)rows * (double)C, each = (double)((rows + sms - 1) / sms);
+  const double direct = 4.5e-6 * weights + (outliers ? 1.3 + 0.35e-3 * std::min((double)rows, 8000.0) : 0.0);
+  const double tile = 0.6 + each * std::max(0.115, 0.07 + 0.23e-3 * (double)C) + 0.13 * std::min(each, 40.0);
+  return weights > (outliers ? 1500.0 : 16384.0) && direct > tile;
+}
+
+// The kernel's dynamic shared-memory limit is a per-device attribute: set once
+// per device, and again if a launch reports an invalid configuration (the
+// device's context may have been reset since).
+static cudaError_t launch_tile(const LayerArgs &p, int64_t row0, int64_t nrows, float *W, const DecLayout &lay, int dev,
+                               int grid, cudaStream_t st) {
+  static DeviceOnce once;
+  auto limit = [&] {
+    return (cudaError_t)once.run(dev, [] {
+      return (int)cudaFuncSetAttribute(k_decode_tile, cudaFuncAttributeMaxDynamicSharedMemorySize, kDecSmemMax);
+    });
+  };
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(kDecThreads + 32);
+  cfg.dynamicSmemBytes = lay.total;
+  cfg.stream = st;
+  cudaError_t e = limit();
+  if (e == cudaSuccess) e = cudaLaunchKernelEx(&cfg, k_decode_tile, p, row0, nrows, W, lay);
+  if (e == cudaErrorInvalidValue) {
+    (void)cudaGetLastError();
+    once.forget(dev);
+    e = limit();
+    if (e == cudaSuccess) e = cudaLaunchKernelEx(&cfg, k_decode_tile, p, row0, nrows, W, lay);
+  }
+  return e;
+}
+
 }  // namespace seedq
 
 using namespace seedq;
@@ -398,7 +443,8 @@ seedq_status seedq_decode_rows(const seedq_layer *L, int64_t row0, int64_t nrows
   const int64_t C = L->args.C;
   DecLayout lay = dec_layout(C, 1, 2);
   if (lay.total > (uint32_t)kDecSmemMax) lay = dec_layout(C, 1, 1);
-  if (((uintptr_t)W & 15u) == 0 && lay.total <= (uint32_t)kDecSmemMax) {
+  if (((uintptr_t)W & 15u) == 0 && lay.total <= (uint32_t)kDecSmemMax &&
+      tile_is_faster(nrows, C, sms, L->args.n_out > 0)) {
     // Rows per tile: as many as fit twice, fewer when each SM would get less
     // than four tiles, but at least a chunk for every decoding warp while that
     // leaves each SM a tile.
@@ -411,10 +457,7 @@ seedq_status seedq_decode_rows(const seedq_layer *L, int64_t row0, int64_t nrows
       if (rows > 1) lay = dec_layout(C, (int)rows, 2);
     }
     const int64_t tiles = (nrows + lay.trows - 1) / lay.trows;
-    // Per call: the attribute belongs to the current device.
-    SEEDQ_CUDA(cudaFuncSetAttribute(k_decode_tile, cudaFuncAttributeMaxDynamicSharedMemorySize, kDecSmemMax));
-    k_decode_tile<<<(int)(tiles < sms ? tiles : sms), kDecThreads + 32, lay.total, st>>>(L->args, row0, nrows, W, lay);
-    SEEDQ_CUDA(cudaGetLastError());
+    SEEDQ_CUDA(launch_tile(L->args, row0, nrows, W, lay, dev, (int)(tiles < sms ? tiles : sms), st));
     return SEEDQ_OK;
   }
   const int64_t blocks = nrows * (int64_t)L->args.nb;
