@@ -30,6 +30,7 @@
 
 #include "cp_async.cuh"
 #include "device_once.h"
+#include "short_rounds.h"
 #include "f32x2.cuh"
 #include "seedq_internal.cuh"
 
@@ -746,24 +747,16 @@ static cudaError_t launch_fused_as(const cudaLaunchConfig_t &cfg, const MultiArg
 }
 
 // Launches of short rounds take the kernel that fits the stage width to the
-// round: at full width a round of 27 columns (1024 x 1024 at b1) keeps one warp
-// of twelve busy.  A round wide enough for half the warps gains nothing from
-// more of them, and the narrower stages cost it.  With several tensors some
-// CTAs have a round on each side of a tensor's end, and those finish last:
-// there the line is a whole stage per warp.  For n >= 2 (narrower stages, more
-// to stage per column) it lies at a quarter of the warps.  Measured, full width
-// / fitted, us: b1 1024 x 1024 14.5 / 12.5, 64 x 11008 20.0 / 17.2, 2048 x 2816
-// 16.5 / 16.5, 5120 x 2048 20.4 / 20.6, a d = 1024 layer 28.8 / 24.9; b4 512 x
-// 1024 16.0 / 14.5, 64 x 11008 30.8 / 26.9, 2048 x 1024 16.5 / 16.5, 4096 x 1024
-// 16.6 / 18.6.
+// round (short_rounds.h).
+// R, nb: of a single tensor.
 template <int NB, bool kSet>
-static cudaError_t launch_fused(const cudaLaunchConfig_t &cfg, const MultiArgs &a, int64_t units) {
+static cudaError_t launch_fused(const cudaLaunchConfig_t &cfg, const MultiArgs &a, int64_t units, int64_t R, int nb) {
   if constexpr (on_tensor_cores(NB)) {
     return launch_fused_as<NB, kSet, false>(cfg, a);
   } else {
-    const int64_t full = (int64_t)a.ctas * (Cfg<NB>::ST * kWarps);
-    const int64_t line = NB > 1 ? full / 4 : a.nt > 1 ? full : full / 2;
-    return units < line ? launch_fused_as<NB, kSet, true>(cfg, a) : launch_fused_as<NB, kSet, false>(cfg, a);
+    return short_rounds(NB, units, a.ctas, Cfg<NB>::ST * kWarps, a.nt, R, nb)
+               ? launch_fused_as<NB, kSet, true>(cfg, a)
+               : launch_fused_as<NB, kSet, false>(cfg, a);
   }
 }
 
@@ -939,7 +932,7 @@ static seedq_status launch(const seedq_layer *const *layers, int nt, const uint1
       attr[0].val.programmaticStreamSerializationAllowed = 1;
       cfg.attrs = attr;
       cfg.numAttrs = 1;
-      e = launch_fused<NB, false>(cfg, *a, a->cta_begin[a->ctas]);
+      e = launch_fused<NB, false>(cfg, *a, a->cta_begin[a->ctas], layers[0]->args.R, layers[0]->args.nb);
     }
     if (e != cudaSuccess) rc = cuda_fail(e);
   }
@@ -1013,7 +1006,7 @@ static seedq_status launch_set(const seedq_layer_set *S, const uint16_t *X, int 
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    e = launch_fused<NB, true>(cfg, a, S->units);
+    e = launch_fused<NB, true>(cfg, a, S->units, S->rpre[1], (int)(S->cpre[1] / 8));
   }
   return e == cudaSuccess ? SEEDQ_OK : cuda_fail(e);
 }
