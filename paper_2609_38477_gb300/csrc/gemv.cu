@@ -777,17 +777,20 @@ constexpr double kMmSnap = 20.0;
 // Cost-balanced ranges of the units of all tensors, one per CTA.  A group's
 // cost is its modeled time at batch n (block passes and the sum of k over
 // them); inside the group where a range is cut, the first row's rung profile,
-// scaled to the group's cost, places the cut.  One sweep over the groups
-// places all cuts in order.
+// scaled to the group's cost, places the cut.  The cuts are placed in order,
+// each group found from where its tensor's cost would put it if it rose evenly
+// (a look at all 4008 groups of a 128256-row head took a call 7 us).
 static void partition(const seedq_layer *const *layers, int nt, int n, int64_t *ubegin, int64_t *cta_begin,
                       int &ctas_out) {
   // A unit's rows: one group of 32, or a superblock of them on the tensor cores.
   const int gs = on_tensor_cores(batch_template(n)) ? kMmGroups : 1;
   const double cb = cost_block(n);
   auto groups = [&](const seedq_layer *L) { return ((L->args.R + 31) / 32 + gs - 1) / gs; };
-  auto gcost = [&](const seedq_layer *L, int64_t g) {
-    const int64_t i = std::min(g * gs, (L->args.R + 31) / 32);
-    return gs > 1 ? kCostK * L->h_mk[i] + cb * L->h_mp[i] : kCostK * L->h_gk[i] + cb * L->h_gp[i];
+  // Cost of a tensor before unit row g of G.
+  auto cost_before = [&](const seedq_layer *L, int64_t g, int64_t G) {
+    const double *k = gs > 1 ? L->h_mk : L->h_gk, *p = gs > 1 ? L->h_mp : L->h_gp;
+    const int64_t i = g == G ? (L->args.R + 31) / 32 : g * gs;
+    return kCostK * k[i] + cb * p[i];
   };
   int64_t U = 0, sbs = 0;
   double total = 0.0;
@@ -797,7 +800,7 @@ static void partition(const seedq_layer *const *layers, int nt, int n, int64_t *
     ubegin[i] = U;
     sbs += G;
     U += G * L->args.nb;
-    total += gcost(L, G);
+    total += cost_before(L, G, G);
   }
   int ctas = layers[0]->max_ctas;
   if (ctas > kMaxCtas) ctas = kMaxCtas;
@@ -812,10 +815,30 @@ static void partition(const seedq_layer *const *layers, int nt, int n, int64_t *
     const seedq_layer *L = layers[ti];
     const int64_t G = groups(L);
     const int J = L->args.J, Jm1 = J > 1 ? J - 1 : 1, nb = L->args.nb;
-    for (int64_t g = 0; g < G && c < ctas; ++g) {
-      const double g0 = gcost(L, g), g1 = gcost(L, g + 1);
+    const double cost = cost_before(L, G, G);
+    int64_t g = 0;
+    while (c < ctas) {
       double target = total * c / ctas;
-      if (target - tbase >= g1) continue;
+      if (target - tbase >= cost) break;
+      // The first group, from g on, that ends past the target.
+      const double at_cut = target - tbase;
+      auto past = [&](int64_t i) { return cost_before(L, i + 1, G) > at_cut; };
+      int64_t lo = g, hi = G - 1, step = 1;
+      const int64_t guess = std::max(lo, std::min(hi, (int64_t)(at_cut / cost * (double)G)));
+      if (past(guess)) {
+        for (hi = guess; hi - step >= lo && past(hi - step); step *= 2) hi -= step;
+        lo = std::max(lo, hi - step + 1);
+      } else {
+        for (lo = guess + 1; lo + step <= hi && !past(lo + step - 1); step *= 2) lo += step;
+        hi = std::min(hi, lo + step - 1);
+      }
+      while (lo < hi) {
+        const int64_t mid = (lo + hi) >> 1;
+        if (past(mid)) hi = mid;
+        else lo = mid + 1;
+      }
+      g = lo;
+      const double g0 = cost_before(L, g, G), g1 = cost_before(L, g + 1, G);
       const int32_t *b = L->h_repbk + g * gs * Jm1;
       double rep = 0.0;
       for (int j = 0, clo = 0; j < J; ++j) {
@@ -866,7 +889,7 @@ static void partition(const seedq_layer *const *layers, int nt, int n, int64_t *
         target = total * c / ctas;
       }
     }
-    tbase += gcost(L, G);
+    tbase += cost;
   }
   // Cuts left over by rounding at the very end of the sequence.
   for (; c < ctas; ++c) {
