@@ -263,8 +263,9 @@ uint32_t seedq_lfsr_taps(int32_t S);
  * Outputs per block b: seed[b] (uint32), E[b] (int8), t[6 b + j] (int8, j < k;
  * the rest 0), err[b] (double; may be NULL).  All device pointers; work is
  * enqueued on cuda_stream, with scratch allocated and freed in stream order
- * (seeds are screened before they are evaluated); a call that can get none
- * evaluates every seed, with the same results and far more slowly. */
+ * (seeds are screened before they are evaluated); a call for which the device
+ * has no memory left evaluates every seed, with the same results and up to 500
+ * times as slowly.  Other failures of the allocation are SEEDQ_ERR_CUDA. */
 
 /* Blocks at one rung (S even in 8..16, k in 2..6): w is device nblocks x 8
  * float32, row-major (one block per row).  Other rungs: SEEDQ_ERR_UNSUPPORTED. */

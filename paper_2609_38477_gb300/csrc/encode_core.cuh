@@ -335,8 +335,9 @@ __device__ __forceinline__ void gather_block(const LayerArgs &p, const float *W,
   }
 }
 
-// Screened search (encode_screen.cu).  False when its scratch could not be
-// had: nothing was launched, and the caller takes the exhaustive kernels.
+// Screened search (encode_screen.cu).  False when there was no memory for its
+// scratch: nothing was launched, and the caller takes the exhaustive kernels.
+// Any other failure is in *e.
 bool screen_blocks(int S, int K, const float *w, int64_t nblocks, const EncodeOut &o, cudaStream_t st,
                    cudaError_t *e);
 bool screen_layer(const seedq_layer *L, const float *W, const EncodeOut &o, cudaStream_t st, cudaError_t *e);

@@ -880,11 +880,9 @@ bool screen(ScreenArgs &a, const LayerArgs &p, cudaStream_t st, cudaError_t *e) 
   const size_t arrive = sc.take(zeroed);
   const size_t wide = sc.take(4 * (size_t)table_ctas * kTableThreads);
   *e = cudaMallocAsync((void **)&sc.base, sc.bytes, st);
-  if (*e != cudaSuccess) {
-    (void)cudaGetLastError();
-    *e = cudaSuccess;
-    return false;
-  }
+  if (*e != cudaSuccess) (void)cudaGetLastError();
+  if (*e == cudaErrorMemoryAllocation) return false;
+  if (*e != cudaSuccess) return true;  // not a lack of memory: the caller reports it
   for (int j = 0; j < a.njobs; ++j) {
     a.job[j].tab = SeedTables{reinterpret_cast<uint2 *>(sc.base + frag[j]),
                               reinterpret_cast<uint32_t *>(sc.base + mask[j]),
