@@ -263,10 +263,19 @@ __global__ void __launch_bounds__(kDecThreads + 32, 1)
       __syncwarp();
     };
     for (int b = 0; b < kDecStages; ++b) stage(blockIdx.x + (int64_t)b * gridDim.x, b);
-    uint32_t b = 0, ph = 0, sb = 0;
+    uint32_t b = 0, ph = 0, sb = 0, sph = 0;
     for (int64_t tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
       if (!mbar_wait(F.full + b, ph)) {
+        // The decoding warps have given up.  Copies into this CTA's shared
+        // memory must not outlive it: those of the kDecStages tiles from here.
         atomicOr(p.flags, 1u);
+        for (int k = 0; k < kDecStages && tile + (int64_t)k * gridDim.x < tiles; ++k) {
+          mbar_wait(F.ready + sb, sph);
+          if (++sb == kDecStages) {
+            sb = 0;
+            sph ^= 1;
+          }
+        }
         break;
       }
       if (t == kDecThreads) {
@@ -282,7 +291,10 @@ __global__ void __launch_bounds__(kDecThreads + 32, 1)
         asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
         mbar_arrive(F.free_ + b);
       }
-      sb = sb + 1 == kDecStages ? 0 : sb + 1;
+      if (++sb == kDecStages) {
+        sb = 0;
+        sph ^= 1;
+      }
       if (++b == (uint32_t)nbuf) {
         b = 0;
         ph ^= 1;
