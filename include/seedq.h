@@ -238,8 +238,11 @@ seedq_status seedq_layer_row_offsets(const seedq_layer *layer, uint64_t *offsets
  * the readable bytes of the stream (the read is cut off there, the affected
  * weights or rows are wrong, nothing outside the buffer is read), or the bits a
  * row's blocks occupy by its rung breakpoints differ from its row offsets.
- * Never set for a stream bound with seedq_layer_bind_stream and a plan from
- * seedq_layer_prepare.  Synchronous; 0 means no fault was seen. */
+ * Never set for that reason for a stream bound with seedq_layer_bind_stream and
+ * a plan from seedq_layer_prepare.  The full decode also sets bit 0 when one of
+ * its bounded waits for a copy runs out (a second or so: the device did not
+ * make progress); the rest of that call's output is then not written.
+ * Synchronous; 0 means no fault was seen. */
 seedq_status seedq_last_device_error(const seedq_layer *layer, uint32_t *flags);
 
 /* Tap mask T_S of the width-S LFSR used by the stream format (bit i set when
