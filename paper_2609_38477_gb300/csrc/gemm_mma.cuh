@@ -54,6 +54,7 @@ constexpr int kMmRows = 32 * kMmGroups;
 
 template <int NB>
 struct MmCfg {
+  static_assert(NB == 8 || NB == 16, "smaller batches run on the FMA pipes");
   static constexpr int ST = 24;                   // columns per stage
   static constexpr int ACC = NB == 16 ? 16 : 8;   // sums a lane holds
   static constexpr int XW = ST * kMmParts;        // columns per window
@@ -124,7 +125,7 @@ __device__ __forceinline__ void mm_cols(const uint4 *rent, const uint32_t *rows,
     uint32_t xv[NB == 16 ? 2 : 1][8];
     {
       const uint8_t *xp = xs + min(col, chi - 1) * CF::XCOL + g * 16;
-      const bool in = (!kUni || col < chi) && (NB >= 8 || g < NB);
+      const bool in = !kUni || col < chi;
 #pragma unroll
       for (int t = 0; t < (NB == 16 ? 2 : 1); ++t) {
         uint4 v = make_uint4(0u, 0u, 0u, 0u);
@@ -649,7 +650,7 @@ __global__ void __launch_bounds__(kMmThreads, 1) k_gemm(const __grid_constant__ 
           cr[8] = tot[4 * s + 2];
           cr[NB + 8] = tot[4 * s + 3];
         }
-      } else if (NB >= 8 || q < NB / 2) {  // batch 2q and 2q + 1 of rows 16h + g and 16h + g + 8
+      } else {  // batch 2q and 2q + 1 of rows 16h + g and 16h + g + 8
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
           float *cr = cg + (16 * h + g) * NB + 2 * q;
