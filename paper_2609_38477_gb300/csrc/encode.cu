@@ -41,16 +41,11 @@ namespace seedq {
 constexpr int kEncWarps = 8;
 
 // Whether a call takes the screened search (encode_screen.cu).  Its tables and
-// thresholds are a fixed cost (about 150 us), which 255 seeds, or 1023 of two
-// coefficients, do not repay on small calls.  Measured, exhaustive / screened, us:
-// (8, 2) 110 / 170 at 2048 blocks, 201 / 192 at 4000; (8, 3) 165 / 197, 303 / 195;
-// (8, 4) 165 / 215 at 1000, 299 / 215 at 2048; (8, 5) 239 / 260, 461 / 285; (8, 6)
-// 268 / 230 at one block, 343 / 350 at 1000, 660 / 340 at 2048; (10, 2) 134 / 150 at
-// one block, 173 / 160 at 20; (10, 3) 217 / 160 at one block.
-static bool screened(int S, int K, int64_t nblocks) {
-  if (S == 8) return nblocks > (K <= 3 ? 2048 : K == 4 ? 1300 : K == 5 ? 1100 : 0);
-  return S > 10 || K > 2 || nblocks > 15;
-}
+// thresholds are a fixed cost (about 150 us), which 255 seeds of few
+// coefficients do not repay on small calls; measured at (8, 3), exhaustive
+// against screened: 84 / 163 us at 100 blocks, 162 / 182 at 2000, 1214 / 194
+// at 20000; at (8, 6) 340 / 322 at 100; at (10, 2) 176 / 164 at 100.
+static bool screened(int S, int K, int64_t nblocks) { return S > 8 || K > 3 || nblocks > 2048; }
 
 // Search all seeds of one block (w: 8 weights) for the lane's share of seeds.
 // Returns the lane's best (error, seed, E, t) in the order of the scan.
