@@ -41,10 +41,14 @@ namespace seedq {
 constexpr int kEncWarps = 8;
 
 // Whether a call takes the screened search (encode_screen.cu).  Its tables and
-// thresholds are a fixed cost (about 150 us), which 255 seeds of few
-// coefficients do not repay on small calls; measured at (8, 3), exhaustive
-// against screened: 84 / 163 us at 100 blocks, 162 / 182 at 2000, 1214 / 194
-// at 20000; at (8, 6) 340 / 322 at 100; at (10, 2) 176 / 164 at 100.
+// thresholds are a fixed cost (40 to 60 us among other calls; about 150 us more
+// for a call after a synchronization, which finds the scratch given back), which
+// 255 seeds of few coefficients do not repay on small calls.  Measured among other
+// calls, exhaustive / screened, us: (8, 2) 50 / 59 at 100 blocks, 101 / 69 at 2048;
+// (8, 3) 75 / 72, 154 / 82; (8, 4) 91 / 61 at one block, 155 / 102 at 1000; (8, 6)
+// 263 / 116, 332 / 229; (10, 2) 125 / 46, 189 / 70.  Alone: (8, 2) 65 / 231 at 100,
+// 205 / 245 at 4000; (8, 3) 90 / 245, 307 / 255; (8, 4) 107 / 231 at one block, 169 /
+// 272 at 1000, 306 / 275 at 2048; (8, 6) 347 / 406 at 1000.
 static bool screened(int S, int K, int64_t nblocks) { return S > 8 || K > 3 || nblocks > 2048; }
 
 // Search all seeds of one block (w: 8 weights) for the lane's share of seeds.

@@ -447,9 +447,10 @@ __host__ __device__ constexpr int group_cost(int K) { return K == 2 ? 2 : K == 3
 // first) and, within a rung, split by split: a later range of a tile then
 // starts from the errors the earlier ones found.
 __device__ void plan_items(TileState &T, const ScreenArgs &a, int64_t R, int64_t ctas) {
-  int64_t total = 0;
+  int64_t total = 0, all = 0;
   for (int j = 0; j < a.njobs; ++j) {
     T.count[j] = block_count(a, j, R);
+    all += (T.count[j] + kTile - 1) / kTile;
     total += (T.count[j] + kTile - 1) / kTile * (((1 << a.job[j].S) >> 4) * group_cost(a.job[j].K));
   }
   const int64_t target = total / (3 * ctas) + 1;
@@ -459,7 +460,18 @@ __device__ void plan_items(TileState &T, const ScreenArgs &a, int64_t R, int64_t
     const int groups = (1 << a.job[j].S) >> 4;
     const int64_t tiles = (T.count[j] + kTile - 1) / kTile, cost = (int64_t)groups * group_cost(a.job[j].K);
     int64_t s = (cost + target / 2) / target;
-    s = s > groups / 16 ? groups / 16 : s;
+    // With tiles for half the CTAs or more, ranges of 16 groups at least; with
+    // fewer, of eight, with one for sixteen of four (of two at S = 8), where the
+    // evaluations of weights that no seed stands out for (too small or too large
+    // for any exponent) would keep few CTAs busy: 4000 blocks of standard deviation
+    // 1e-4 at (8, 4) 1903 -> 369 us, 1000 at (10, 4) 1760 -> 579; of 0.02 (8, 4) x
+    // 1000 128 -> 103, (10, 2) x 4000 87 -> 90.
+    int most = groups / 16;
+    if (2 * all <= ctas) {
+      const int fine = groups == 16 ? groups / 2 : 16 * all <= ctas ? groups / 4 : groups / 8;
+      most = fine < 64 ? fine : most > 64 ? most : 64;
+    }
+    s = s > most ? most : s;
     if (s < 1 || sitem + tiles * s > a.max_split) s = 1;  // the records are that many
     T.splits[i] = (int)s;
     T.item0[i] = item;
@@ -855,7 +867,7 @@ template <bool kLayer>
 bool screen(ScreenArgs &a, const LayerArgs &p, cudaStream_t st, cudaError_t *e) {
   const int ctas = 2 * sm_count();
   // plan_items makes at most 3 items per CTA and half a tile's worth of
-  // rounding more, and at most one per 16 groups of a tile.
+  // rounding more, and at most 256 of a tile.
   const int64_t tiles = (kLayer ? p.R * (int64_t)p.nb : a.nblocks) / kTile + a.njobs;
   a.max_split = tiles * 256 < 6 * (int64_t)ctas ? tiles * 256 : 6 * (int64_t)ctas;
   Scratch sc;
