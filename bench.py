@@ -928,20 +928,24 @@ def allocate_arm(args):
     for _ in range(max(args.warmup, 3)):
         got = step()
     assert list(got[0]) == d["theta"] and [int(x) for x in got[3]] == d["tie_count"]
-    # Latency of a bisection step driven from the host: a launch, an 8-byte
-    # read-back and a synchronization (the device runs the steps without them).
-    one = torch.zeros(1, dtype=torch.int16, device="cuda")
-    host = torch.zeros(1, dtype=torch.int16, pin_memory=True)
-    for _ in range(20):
-        Q.synth_fp16(0, 0, 1, 1, 0, one)
-        host.copy_(one, non_blocking=True)
-        torch.cuda.synchronize()
-    t0 = time.perf_counter()
-    for _ in range(200):
-        Q.synth_fp16(0, 0, 1, 1, 0, one)
-        host.copy_(one, non_blocking=True)
-        torch.cuda.synchronize()
-    rt = (time.perf_counter() - t0) / 200
+    # The searches' rounds are launches that each wait for the last one: time of
+    # such a launch with next to nothing in it, back to back in a graph.
+    one = torch.zeros(8, dtype=torch.int16, device="cuda")
+    chain = 200
+    Q.synth_fp16(0, 0, 1, 1, 0, one)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        for _ in range(chain):
+            Q.synth_fp16(0, 0, 1, 1, 0, one)
+    rt = float("inf")
+    for _ in range(10):
+        ev = [torch.cuda.Event(enable_timing=True) for _ in range(2)]
+        ev[0].record()
+        graph.replay()
+        ev[1].record()
+        ev[1].synchronize()
+        rt = min(rt, ev[0].elapsed_time(ev[1]) * 1e-3 / chain)
     clocks = Clocks(gpu_index(local))
     dist_barrier()
     clocks.start()
@@ -952,16 +956,14 @@ def allocate_arm(args):
         times.append(time.perf_counter() - t0)
     clk = clocks.stop()
     step_s = dist_max(statistics.mean(times))
-    # Evaluations: the floor's and the multiplier's bisections over 64-bit
-    # patterns, plus the two end points, the tied group and the demotion counts.
-    evals = 64 + 64 + 5
     # Launches: two rankings, the factors, two searches in rounds of up to 31
     # points (as many as keep a round near 2^16 row searches), group and tail.
     rows, probes = sum(R if rho is not None else 1 for R, C, a, rho in factors), 31
     while probes > 1 and rows * probes > 1 << 16:
         probes //= 2
     per_round = (probes + 1).bit_length() - 1
-    launches = 3 + 2 * ((63 + per_round - 1) // per_round + 1) + 2
+    rounds = 2 * ((63 + per_round - 1) // per_round + 1)
+    launches = 3 + rounds + 2
     line = {
         "metric": ALLOC_METRIC, "value": world / step_s, "unit": "allocations/s",
         "n_gpus": world, "steps": args.steps, "warmup": max(args.warmup, 3),
@@ -976,11 +978,11 @@ def allocate_arm(args):
                                           for R, C, a, rho in factors),
                 "d2h_bytes_per_step": 8 * (2 * len(factors) + 47)},
         "gpu_launches": args.steps * launches,
-        "roofline": {"bound": "latency", "achieved": evals / step_s, "peak": 1.0 / rt,
-                     "unit": "dependent evaluations/s", "frac": rt * evals / step_s,
+        "roofline": {"bound": "latency", "achieved": rounds / step_s, "peak": 1.0 / rt,
+                     "unit": "dependent rounds/s", "frac": rt * rounds / step_s,
                      "traffic": None, "kernel": "k_alloc_round (several points a launch)",
-                     "peak_basis": "measured launch + 8-byte read-back + synchronize round trip "
-                                   f"({rt * 1e6:.1f} us); above 1: the searches stay on the device"},
+                     "peak_basis": "measured back-to-back dependent launches of a one-element kernel "
+                                   f"({rt * 1e6:.2f} us each)"},
     }
     if rank == 0 and not args.no_cpu_baseline:
         t = allocate_oracle(args.workload, w, d)
