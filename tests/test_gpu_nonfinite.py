@@ -117,3 +117,42 @@ def test_time_of_a_call(n, bad):
 
     assert time(x) < 5 * time(fin)
     L.release()
+
+
+@pytest.mark.parametrize("n", [7, 16])
+def test_several_tensors_and_sets(n):
+    """One launch over three tensors and a layer set of them, whole and cut
+    superblocks: the outputs of each tensor's own call, NaN for NaN."""
+    from paper_2609_38477_gb300 import seedq as Q
+
+    ts = [_layer(R, C, RUNGS, THETA, n_out, seed, weights=False) for R, C, n_out, seed in
+          ((300, 520, 2, 3), (4100, 64, 0, 4), (40, 2056, 0, 5))]
+    xs = []
+    for i, (L, _, _) in enumerate(ts):
+        x = torch.randn((n, L.cols), generator=torch.Generator(device="cuda").manual_seed(i), device="cuda").to(torch.bfloat16)
+        x[1, 7], x[2, :9], x[4, L.cols - 1], x[n - 1, 3] = float("inf"), float("-inf"), float("nan"), float("-inf")
+        xs.append(x)
+    own = []
+    for (L, _, _), x in zip(ts, xs):
+        y = torch.zeros((n, L.rows), device="cuda")
+        L.gemm_small_batch(x, n, y)
+        own.append(y)
+    multi = [torch.zeros_like(y) for y in own]
+    Q.gemm_multi([t[0] for t in ts], xs, n, multi)
+    S = Q.LayerSet([t[0] for t in ts])
+    Y = torch.zeros(n * sum(t[0].rows for t in ts), device="cuda")
+    S.gemm(torch.cat([x.flatten() for x in xs]), n, Y)
+    torch.cuda.synchronize()
+    for i, y in enumerate(own):
+        # (Each within the bound of tests/test_gpu_gemm.py of the exact product.)
+        Wm = torch.empty((ts[i][0].rows, ts[i][0].cols), device="cuda")
+        ts[i][0].decode_weights(Wm)
+        mag = torch.nan_to_num(xs[i].double(), 0.0, 0.0, 0.0).abs() @ Wm.double().abs().T
+        part = Y[n * int(S.row_offsets[i]):n * int(S.row_offsets[i + 1])].view(n, -1)
+        for other in (multi[i], part):
+            bad = ~torch.isfinite(y)
+            assert bad[[1, 2, 4, n - 1]].all() and not bad[[0, 3]].any()
+            assert torch.equal(torch.isnan(y), torch.isnan(other))
+            assert torch.equal(y[torch.isinf(y)], other[torch.isinf(y)])
+            assert ((y - other).double().abs() <= 4e-5 * mag)[~bad].all()
+    S.release()
