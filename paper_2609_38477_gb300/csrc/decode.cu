@@ -91,7 +91,7 @@ __global__ void k_outliers(const __grid_constant__ LayerArgs p, int64_t row0, in
 // Bound by issue (63% of cycles) and the shared-memory pipe (61%: the scatter's
 // eight random words a block, two table lookups, the rung's constants), ahead
 // of the 4 bytes a weight written.  Measured against k_decode on one GB300:
-// 4096 x 11008 with a row factor and four outlier columns 286 -> 72 us (2.8
+// 4096 x 11008 with a row factor and four outlier columns 287 -> 71 us (2.8
 // TB/s of weights and stream), 4096 x 4096 94 -> 32, 1024 x 1040 9.2 -> 7.6,
 // 512 x 20000 64 -> 29.
 // On the way: two 512-thread CTAs per SM with barriers around each tile 88 us;
